@@ -1,7 +1,7 @@
 // hpd_build_meta: per-step int32 bookkeeping tables and the attention work list (device side).
 //
-// On the caller's stream, no host synchronisation.  Steps with up to 4096 documents take one launch
-// (meta_fused_kernel); larger ones three:
+// On the caller's stream, no host synchronisation.  Steps with up to 4096 documents and 65536 slots take one
+// launch (meta_step_kernel); larger ones three:
 //   doc_scan_kernel   exclusive scans over documents (prefix tokens, slots)
 //   compact_kernel    stable compaction of live slots -> row tables, rows-per-document CSR
 //   plan_kernel       split-KV policy + work list for the attention kernel; -1 fill of table tails
@@ -43,38 +43,6 @@ __device__ __forceinline__ int block_excl_scan(int v, int* smem /* THREADS/32 + 
     total = smem[THREADS / 32];
     __syncthreads();
     return res;
-}
-
-// Two block-wide exclusive scans at the price of one: both values (and both totals) are below 2^31, so they share one
-// 64-bit word without carrying into each other.
-template <int THREADS>
-__device__ __forceinline__ void block_excl_scan2(int a, int b, long long* smem /* THREADS/32 + 1 */, int& ea, int& eb, int& ta, int& tb) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const long long v = static_cast<long long>(static_cast<unsigned>(a)) | (static_cast<long long>(b) << 32);
-    long long incl = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const long long t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += t;
-    }
-    if (lane == 31) smem[warp] = incl;
-    __syncthreads();
-    if (warp == 0) {
-        const long long w = (lane < THREADS / 32) ? smem[lane] : 0;
-        long long wi = w;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const long long t = __shfl_up_sync(0xffffffffu, wi, o);
-            if (lane >= o) wi += t;
-        }
-        if (lane < THREADS / 32) smem[lane] = wi - w;
-        if (lane == 31) smem[THREADS / 32] = wi;
-    }
-    __syncthreads();
-    const long long res = incl - v + smem[warp], tot = smem[THREADS / 32];
-    __syncthreads();
-    ea = static_cast<int>(res & 0xffffffffll); eb = static_cast<int>(res >> 32);
-    ta = static_cast<int>(tot & 0xffffffffll); tb = static_cast<int>(tot >> 32);
 }
 
 __global__ void __launch_bounds__(kScanThreads)
@@ -196,8 +164,9 @@ constexpr int kMinCand = 2;          // smallest chunk size taken: 128 << 2 toke
 
 __device__ __forceinline__ int chunks_of(int L, int cand) {
     if (cand == kCand - 1 || L <= 0) return 1;
-    const int S = kTileN << cand;
-    return (L + S - 1) / S;
+    constexpr int kShift = 7;                           // kTileN = 1 << 7
+    static_assert(kTileN == 1 << kShift, "chunk sizes are powers of two");
+    return static_cast<int>((static_cast<long long>(L) + (kTileN << cand) - 1) >> (kShift + cand));
 }
 
 // Longest units first.  The attention kernel hands units out in list order, a few per pipeline, so a long unit drawn
@@ -218,120 +187,157 @@ __device__ __forceinline__ int unit_cost(int keys, int branch_rows, int G) {
     return min(kUnitCost + keys + branch_rows * G * kBranchCost, static_cast<int>(kCostMax));
 }
 
-template <int THREADS>
-__device__ __forceinline__ void sort_keys_ascending(uint32_t* key, int n2 /* power of two */)
+// Bitonic sort by 1024 threads, ascending.  A thread holds the keys t and t + 1024 in registers: distances below 32 go
+// through shuffles and 1024 through the thread itself, only 32..512 through shared memory (15 of the 55 stages of 1024
+// keys; with every stage in shared memory behind a barrier of its own the sort was half of the table kernel's time).
+// key: n2 keys (n2 a power of two, at most 2048); on return rank[key & 0xFFF] = place for the first n_items keys.
+__device__ __forceinline__ uint32_t bitonic_keep(uint32_t mine, uint32_t other, int i, int j, int k)
 {
-    for (int k = 2; k <= n2; k <<= 1) {
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int t = threadIdx.x; t < n2 / 2; t += THREADS) {
-                const int lo = ((t & ~(j - 1)) << 1) | (t & (j - 1));
-                const int hi = lo + j;
-                const uint32_t a = key[lo], b = key[hi];
-                const bool up = (lo & k) == 0;
-                if ((a > b) == up) { key[lo] = b; key[hi] = a; }
-            }
-            __syncthreads();
-        }
-    }
+    const bool low = (i & j) == 0, up = (i & k) == 0;
+    return low == up ? min(mine, other) : max(mine, other);
 }
 
-// The split-KV plan, run by ONE block of THREADS threads (doc_active_start must be complete and visible).  scratch: kPlanScratchInts ints of shared memory, rank: kSortItems entries.
-template <int THREADS>
+__device__ __forceinline__ void rank_keys(uint32_t* key, int n2, int n_items, uint16_t* rank)
+{
+    const int t = threadIdx.x;
+    const bool two = n2 > 1024;
+    uint32_t e0 = t < n2 ? key[t] : 0xFFFFFFFFu, e1 = two ? key[t + 1024] : 0xFFFFFFFFu;
+    for (int k = 2; k <= n2; k <<= 1) {
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            if (j == 1024) {
+                const uint32_t a = e0, b = e1;
+                e0 = bitonic_keep(a, b, t, j, k);
+                e1 = bitonic_keep(b, a, t + 1024, j, k);
+            } else {
+                uint32_t o0, o1 = 0;
+                if (j < 32) {
+                    o0 = __shfl_xor_sync(0xffffffffu, e0, j);
+                    if (two) o1 = __shfl_xor_sync(0xffffffffu, e1, j);
+                } else {
+                    __syncthreads();                     // the previous exchange has been read
+                    if (t < n2) key[t] = e0;
+                    if (two) key[t + 1024] = e1;
+                    __syncthreads();
+                    o0 = t < n2 ? key[t ^ j] : 0xFFFFFFFFu;
+                    if (two) o1 = key[(t ^ j) + 1024];
+                }
+                e0 = bitonic_keep(e0, o0, t, j, k);
+                if (two) e1 = bitonic_keep(e1, o1, t + 1024, j, k);
+            }
+        }
+    }
+    __syncthreads();                                     // rank may share memory with nothing, but its readers wait here
+    if (t < n_items) rank[e0 & 0xFFFu] = static_cast<uint16_t>(t);
+    if (two && t + 1024 < n_items) rank[e1 & 0xFFFu] = static_cast<uint16_t>(t + 1024);
+    __syncthreads();
+}
+
+// Block-wide exclusive scan of one 64-bit word per thread (two packed ints) by 1024 threads behind ONE barrier: every warp
+// scans the 32 warp totals for itself.  buf alternates between consecutive calls.
+__device__ __forceinline__ long long scan_words(long long v, long long* buf, long long& total)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    long long incl = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const long long u = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += u;
+    }
+    if (lane == 31) buf[warp] = incl;
+    __syncthreads();
+    const long long w = buf[lane];
+    long long wi = w;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const long long u = __shfl_up_sync(0xffffffffu, wi, o);
+        if (lane >= o) wi += u;
+    }
+    total = __shfl_sync(0xffffffffu, wi, 31);
+    return incl - v + __shfl_sync(0xffffffffu, wi - w, warp);
+}
+__device__ __forceinline__ long long words(int lo, int hi) { return static_cast<long long>(static_cast<unsigned>(lo)) | (static_cast<long long>(hi) << 32); }
+__device__ __forceinline__ int word_lo(long long v) { return static_cast<int>(v & 0xffffffffll); }
+__device__ __forceinline__ int word_hi(long long v) { return static_cast<int>(v >> 32); }
+
+// The split-KV plan, run by ONE block of 1024 threads; the two document tables may be in shared or global memory.
+// scratch: kPlanScratchInts ints of shared memory, rank: kSortItems entries.
+// A serial chain of barriers and shuffles with little work in between: sums go through warp reductions, one candidate chunk
+// size per warp, and one-barrier scans (the same sums as 64-bit shuffles and shared-memory atomics of all 32 warps took 5 us of
+// the 12 us this kernel needed for a step of few documents).
 __device__ __forceinline__ void plan_block(int n_docs, int G, int Hkv, int n_sm,
                                            const int32_t* doc_prefix_len, const int32_t* doc_active_start,
                                            int* scratch, uint16_t* rank,
                                            WsHeader* __restrict__ hdr, WorkItem* __restrict__ work, DocSplit* __restrict__ split,
                                            int work_cap, int part_cap)
 {
-    constexpr int kPlanThreads = THREADS;
-    __shared__ long long sm2[kPlanThreads / 32 + 1];
-    __shared__ int sm1[kPlanThreads / 32 + 1];
-    __shared__ long long red[kCand * 2];
-    __shared__ int s_choice, s_cost_min, s_cost_max;
-    const int rows_per_block = kTileM / G;
+    __shared__ long long buf[2][32];
+    __shared__ long long s_items[kCand], s_prow[kCand];
+    __shared__ int s_whole, s_cost_min, s_cost_max, s_choice;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int rows_per_block = kTileM / G;               // a power of two
+    const int rb_shift = 31 - __clz(rows_per_block);
+    auto rows_of = [&](int d) { return doc_active_start[d + 1] - doc_active_start[d]; };
+    auto blocks_of = [&](int rows) { return (rows + rows_per_block - 1) >> rb_shift; };
 
     // the usual case first: whole documents already give one unit per SM or more -> nothing to weigh
     // (the same pass weighs the whole documents' units: only lists whose units differ in length are put in order below)
-    if (threadIdx.x < kCand * 2) red[threadIdx.x] = 0;
-    if (threadIdx.x == 0) { s_cost_min = 0x7fffffff; s_cost_max = 0; }
+    if (threadIdx.x == 0) { s_whole = 0; s_cost_min = 0x7fffffff; s_cost_max = 0; }
     __syncthreads();
-    {
-        long long whole = 0;
-        int cmin = 0x7fffffff, cmax = 0;
-        for (int d = threadIdx.x; d < n_docs; d += kPlanThreads) {
-            const int rows = __ldcg(doc_active_start + d + 1) - __ldcg(doc_active_start + d);
+    for (int base = warp * 32; base < n_docs; base += kPlanThreads) {
+        const int d = base + lane;
+        int whole = 0, cmin = 0x7fffffff, cmax = 0;
+        if (d < n_docs) {
+            const int rows = rows_of(d);
             if (rows > 0) {
-                const int mb = (rows + rows_per_block - 1) / rows_per_block;
-                whole += mb;
+                whole = blocks_of(rows);
                 const int L = min(max(doc_prefix_len[d], 0), static_cast<int>(kCostMax));
-                cmin = min(cmin, unit_cost(L, rows - (mb - 1) * rows_per_block, G));
-                cmax = max(cmax, unit_cost(L, min(rows, rows_per_block), G));
+                cmin = unit_cost(L, rows - (whole - 1) * rows_per_block, G);
+                cmax = unit_cost(L, min(rows, rows_per_block), G);
             }
         }
-        for (int o = 16; o > 0; o >>= 1) {
-            whole += __shfl_down_sync(0xffffffffu, whole, o);
-            cmin = min(cmin, __shfl_xor_sync(0xffffffffu, cmin, o));
-            cmax = max(cmax, __shfl_xor_sync(0xffffffffu, cmax, o));
-        }
-        if ((threadIdx.x & 31) == 0 && whole) {
-            atomicAdd(reinterpret_cast<unsigned long long*>(&red[0]), static_cast<unsigned long long>(whole));
-            atomicMin(&s_cost_min, cmin); atomicMax(&s_cost_max, cmax);
-        }
+        whole = __reduce_add_sync(0xffffffffu, whole);
+        cmin = __reduce_min_sync(0xffffffffu, cmin);
+        cmax = __reduce_max_sync(0xffffffffu, cmax);
+        if (lane == 0 && whole) { atomicAdd(&s_whole, whole); atomicMin(&s_cost_min, cmin); atomicMax(&s_cost_max, cmax); }
     }
     __syncthreads();
-    const bool enough = red[0] * Hkv >= n_sm;
+    const bool enough = static_cast<long long>(s_whole) * Hkv >= n_sm;
     // worth the sort only when the units differ: more than a quarter between the shortest and the longest (a split
     // list always goes through the pass below: its chunks differ)
     const bool differ = !enough || (s_cost_max > s_cost_min && (s_cost_max - s_cost_min) * 4 > s_cost_max);
-    __syncthreads();
-    if (enough) {
-        if (threadIdx.x == 0) s_choice = kCand - 1;
-    } else {
-    if (threadIdx.x < kCand * 2) red[threadIdx.x] = 0;
-    __syncthreads();
-    {
-        long long items[kCand], prow[kCand];
-#pragma unroll
-        for (int c = 0; c < kCand; ++c) { items[c] = 0; prow[c] = 0; }
-        for (int d = threadIdx.x; d < n_docs; d += kPlanThreads) {
-            const int rows = __ldcg(doc_active_start + d + 1) - __ldcg(doc_active_start + d);
-            if (rows <= 0) continue;
-            const int mb = (rows + rows_per_block - 1) / rows_per_block;
-            const int L = doc_prefix_len[d];
-#pragma unroll
-            for (int c = 0; c < kCand; ++c) {
-                const int ch = chunks_of(L, c);
-                items[c] += static_cast<long long>(ch) * mb;
-                if (ch > 1) prow[c] += static_cast<long long>(ch) * rows;
+    int cand = kCand - 1;                                // whole documents
+    if (!enough) {
+        if (warp < kCand) {                              // warp c weighs chunk size c
+            long long items = 0, prow = 0;
+            for (int d = lane; d < n_docs; d += 32) {
+                const int rows = rows_of(d);
+                if (rows <= 0) continue;
+                const int ch = chunks_of(doc_prefix_len[d], warp);
+                items += static_cast<long long>(ch) * blocks_of(rows);
+                if (ch > 1) prow += static_cast<long long>(ch) * rows;
             }
-        }
 #pragma unroll
-        for (int c = 0; c < kCand; ++c) {
-            long long a = items[c], b = prow[c];
             for (int o = 16; o > 0; o >>= 1) {
-                a += __shfl_down_sync(0xffffffffu, a, o);
-                b += __shfl_down_sync(0xffffffffu, b, o);
+                items += __shfl_down_sync(0xffffffffu, items, o);
+                prow += __shfl_down_sync(0xffffffffu, prow, o);
             }
-            if ((threadIdx.x & 31) == 0) {
-                atomicAdd(reinterpret_cast<unsigned long long*>(&red[c]), static_cast<unsigned long long>(a));
-                atomicAdd(reinterpret_cast<unsigned long long*>(&red[kCand + c]), static_cast<unsigned long long>(b));
+            if (lane == 0) { s_items[warp] = items; s_prow[warp] = prow; }
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            int c = kCand - 1;
+            while (c > kMinCand && s_items[c] * Hkv < n_sm) {
+                const int nc = c - 1;
+                if (s_items[nc] > work_cap || s_prow[nc] > part_cap) break;
+                c = nc;
             }
+            s_choice = c;
         }
+        __syncthreads();
+        cand = s_choice;
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int c = kCand - 1;                              // whole documents
-        while (c > kMinCand && red[c] * Hkv < n_sm) {
-            const int nc = c - 1;
-            if (red[nc] > work_cap || red[kCand + nc] > part_cap) break;
-            c = nc;
-        }
-        s_choice = c;
-    }
-    }
-    __syncthreads();
-    const int cand = s_choice;
 
+    int parity = 0;
     // ---- order of the list: rank[item in document order] = its place, longest first ----
     bool sorted = false;
     if (n_docs <= kSortDocs && differ) {
@@ -341,12 +347,13 @@ __device__ __forceinline__ void plan_block(int n_docs, int G, int Hkv, int n_sm,
             const int d = base + threadIdx.x;
             int rows = 0, L = 0, mb = 0, ch = 0;
             if (d < n_docs) {
-                rows = __ldcg(doc_active_start + d + 1) - __ldcg(doc_active_start + d);
+                rows = rows_of(d);
                 L = doc_prefix_len[d];
-                if (rows > 0) { mb = (rows + rows_per_block - 1) / rows_per_block; ch = chunks_of(L, cand); }
+                if (rows > 0) { mb = blocks_of(rows); ch = chunks_of(L, cand); }
             }
-            int tot;
-            const int ei = n_items + block_excl_scan<kPlanThreads>(ch * mb, sm1, tot);
+            long long tot;
+            const int ei = n_items + word_lo(scan_words(ch * mb, buf[parity], tot));
+            parity ^= 1;
             if (d < n_docs) {
                 const int S = (cand == kCand - 1) ? L : (kTileN << cand);
                 for (int c = 0, w = ei; c < ch; ++c) {
@@ -358,18 +365,15 @@ __device__ __forceinline__ void plan_block(int n_docs, int G, int Hkv, int n_sm,
                     }
                 }
             }
-            n_items += tot;
+            n_items += word_lo(tot);
         }
-        __syncthreads();
         if (n_items > 1 && n_items <= kSortItems) {
             sorted = true;
             int n2 = 2;
             while (n2 < n_items) n2 <<= 1;
             for (int w = n_items + threadIdx.x; w < n2; w += kPlanThreads) s_key[w] = 0xFFFFFFFFu;
             __syncthreads();
-            sort_keys_ascending<kPlanThreads>(s_key, n2);
-            for (int i = threadIdx.x; i < n_items; i += kPlanThreads) rank[s_key[i] & 0xFFFu] = static_cast<uint16_t>(i);
-            __syncthreads();
+            rank_keys(s_key, n2, n_items, rank);
         }
     }
 
@@ -380,18 +384,14 @@ __device__ __forceinline__ void plan_block(int n_docs, int G, int Hkv, int n_sm,
         const int d = base + threadIdx.x;
         int rows = 0, L = 0, mb = 0, ch = 0;
         if (d < n_docs) {
-            rows = __ldcg(doc_active_start + d + 1) - __ldcg(doc_active_start + d);
+            rows = rows_of(d);
             L = doc_prefix_len[d];
-            if (rows > 0) {
-                mb = (rows + rows_per_block - 1) / rows_per_block;
-                ch = chunks_of(L, cand);
-            }
+            if (rows > 0) { mb = blocks_of(rows); ch = chunks_of(L, cand); }
         }
-        const int my_items = ch * mb;
-        const int my_part = ch > 1 ? ch * rows : 0;
-        int tot_i, tot_p, ei, ep;
-        block_excl_scan2<kPlanThreads>(my_items, my_part, sm2, ei, ep, tot_i, tot_p);
-        ei += run_items; ep += run_part;
+        long long tot;
+        const long long ex = scan_words(words(ch * mb, ch > 1 ? ch * rows : 0), buf[parity], tot);
+        parity ^= 1;
+        const int ei = run_items + word_lo(ex), ep = run_part + word_hi(ex);
         if (d < n_docs) {
             split[d].part_base = ch > 1 ? ep : -1;
             split[d].n_chunks = ch;
@@ -415,8 +415,8 @@ __device__ __forceinline__ void plan_block(int n_docs, int G, int Hkv, int n_sm,
                 }
             }
         }
-        run_items += tot_i;
-        run_part += tot_p;
+        run_items += word_lo(tot);
+        run_part += word_hi(tot);
     }
     const int split_any = __syncthreads_or(any_split);
     if (threadIdx.x == 0) {
@@ -454,109 +454,125 @@ plan_kernel(int n_docs, int n_slots, int G, int Hkv, int n_sm,
     }
     __shared__ int s_scratch[kPlanScratchInts];
     __shared__ uint16_t s_rank[kSortItems];
-    plan_block<kPlanThreads>(n_docs, G, Hkv, n_sm, doc_prefix_len, doc_active_start, s_scratch, s_rank,
+    plan_block(n_docs, G, Hkv, n_sm, doc_prefix_len, doc_active_start, s_scratch, s_rank,
                              hdr, work, split, work_cap, part_cap);
 }
 
 // ---------------------------------------------------------------------------------------------------------------
-// All of the above in ONE launch, for steps with at most kFusedDocs documents (the usual case).  Every block of 256
-// slots repeats the two cheap global steps for itself -- the scans over documents (kept in shared memory) and the
-// count of live slots before it and in total -- so that it can place its live slots' rows, its dead slots' -1 entries
-// at the tail, and its documents' CSR entries without waiting for any other block.  The block that finishes last
-// (counted in the workspace header) sees every block's CSR entries and writes the split-KV plan.
+// All of the above in ONE launch without any dependency between blocks, for steps of at most kStepDocs documents and
+// kStepSlots slots (the usual case).  The kernel is a chain of memory and barrier latencies, not of bytes, so every block
+// repeats the cheap global steps for itself: the scans over documents, and the live flags of ALL slots as a bit mask with
+// a prefix count per 32 slots, both in shared memory.  From there "live slots before s" is one lookup for any s: the row
+// blocks place their 1024 slots' rows and -1 tail entries with it, and block 0 derives every document's row range and
+// writes the split-KV plan from shared memory alone.  One round trip to memory in all; the earlier form, in which the
+// last row block to finish (a counter in the workspace, cleared by a memset) wrote the plan, took four.
 // ---------------------------------------------------------------------------------------------------------------
-constexpr int kFusedDocs = 4096;
-constexpr int kFusedThreads = 256;
+constexpr int kStepDocs = 4096;
+constexpr int kStepSlots = 65536;                    // two mask words per thread
+constexpr int kStepWords = kStepSlots / 32;
 
-__device__ __forceinline__ int count_alive(const uint8_t* __restrict__ slot_alive, int begin, int end)
-{
-    // live slots in [begin, end), 16 bytes at a time where the address allows
-    int cnt = 0;
-    const uintptr_t addr = reinterpret_cast<uintptr_t>(slot_alive + begin);
-    int head = static_cast<int>((16 - (addr & 15)) & 15);
-    if (head > end - begin) head = end - begin;
-    for (int i = begin + threadIdx.x; i < begin + head; i += blockDim.x) cnt += slot_alive[i] != 0;
-    const int n_vec = (end - begin - head) / 16;
-    const uint4* v = reinterpret_cast<const uint4*>(slot_alive + begin + head);
-    for (int i = threadIdx.x; i < n_vec; i += blockDim.x) {
-        const uint4 w = v[i];
-        cnt += __popc(__vcmpne4(w.x, 0u) & 0x01010101u) + __popc(__vcmpne4(w.y, 0u) & 0x01010101u) +
-               __popc(__vcmpne4(w.z, 0u) & 0x01010101u) + __popc(__vcmpne4(w.w, 0u) & 0x01010101u);
-    }
-    for (int i = begin + head + n_vec * 16 + threadIdx.x; i < end; i += blockDim.x) cnt += slot_alive[i] != 0;
-    return cnt;
+// bit i of the result: byte i of the word is not zero
+__device__ __forceinline__ uint32_t nonzero_bytes(uint32_t w) {
+    return ((__vcmpne4(w, 0u) & 0x08040201u) * 0x01010101u) >> 24;
 }
 
-__global__ void __launch_bounds__(kFusedThreads)
-meta_fused_kernel(int n_docs, int n_slots, int32_t suffix_cap, int32_t pos_gap, int G, int Hkv, int n_sm,
-                  const int32_t* __restrict__ doc_prefix_len, const int32_t* __restrict__ doc_branch_cnt,
-                  const int32_t* __restrict__ slot_depth, const uint8_t* __restrict__ slot_alive,
-                  const int32_t* __restrict__ slot_vis /* nullable */,
-                  int32_t* __restrict__ doc_kv_start, int32_t* __restrict__ doc_slot_start, int32_t* doc_active_start,
-                  int32_t* __restrict__ active_slot, int32_t* __restrict__ doc_id, int32_t* __restrict__ branch_start,
-                  int32_t* __restrict__ pos_id, int32_t* __restrict__ suffix_off, int32_t* __restrict__ suffix_len,
-                  int32_t* __restrict__ prefix_vis /* nullable */,
-                  int32_t* __restrict__ n_active, WsHeader* hdr, WorkItem* __restrict__ work, DocSplit* __restrict__ split,
-                  int work_cap, int part_cap)
+__global__ void __launch_bounds__(kPlanThreads)
+meta_step_kernel(int n_docs, int n_slots, int32_t suffix_cap, int32_t pos_gap, int G, int Hkv, int n_sm,
+                 const int32_t* __restrict__ doc_prefix_len, const int32_t* __restrict__ doc_branch_cnt,
+                 const int32_t* __restrict__ slot_depth, const uint8_t* __restrict__ slot_alive,
+                 const int32_t* __restrict__ slot_vis /* nullable */,
+                 int32_t* __restrict__ doc_kv_start, int32_t* __restrict__ doc_slot_start, int32_t* __restrict__ doc_active_start,
+                 int32_t* __restrict__ active_slot, int32_t* __restrict__ doc_id, int32_t* __restrict__ branch_start,
+                 int32_t* __restrict__ pos_id, int32_t* __restrict__ suffix_off, int32_t* __restrict__ suffix_len,
+                 int32_t* __restrict__ prefix_vis /* nullable */,
+                 int32_t* __restrict__ n_active, WsHeader* __restrict__ hdr, WorkItem* __restrict__ work, DocSplit* __restrict__ split,
+                 int work_cap, int part_cap)
 {
-    __shared__ int sm[kFusedThreads / 32 + 1];
-    __shared__ long long sm2[kFusedThreads / 32 + 1];
-    __shared__ int s_slot_start[kFusedDocs + 1];
-    __shared__ int s_last;
-    const int first = blockIdx.x * kFusedThreads;
-    // this thread's slot: its flags are asked for now and used after the scans
-    const int s = first + threadIdx.x;
-    const int alive = (s < n_slots) && slot_alive[s] != 0;
-    const int depth = s < n_slots ? slot_depth[s] : 0;
-    const int my_vis = (slot_vis && s < n_slots) ? slot_vis[s] : 0;
+    __shared__ int s_start[kStepDocs + 1];           // first slot of every document; block 0 turns it into its first row
+    __shared__ int s_len[kStepDocs];
+    __shared__ uint32_t s_bits[kStepWords + kStepWords / 2];      // live mask, then the 16-bit prefix counts
+    __shared__ long long s_scan[2][32];
+    __shared__ int s_cnt[32];
+    uint32_t* s_mask = s_bits;
+    uint16_t* s_pre = reinterpret_cast<uint16_t*>(s_bits + kStepWords);
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const bool planner = blockIdx.x == 0;
+    const int s = (static_cast<int>(blockIdx.x) - 1) * kPlanThreads + t;
+    const bool mine = !planner && s < n_slots;
 
-    // ---- scans over documents: slot starts stay in shared memory, block 0 also publishes both scans ----
-    {
-        int run_kv = 0, run_sl = 0;
-        for (int base = 0; base < n_docs; base += kFusedThreads) {
-            const int d = base + threadIdx.x;
-            const int l = d < n_docs ? doc_prefix_len[d] : 0;
-            const int c = d < n_docs ? doc_branch_cnt[d] : 0;
-            int tot_l, tot_c, el, ec;
-            block_excl_scan2<kFusedThreads>(l, c, sm2, el, ec, tot_l, tot_c);
-            if (d < n_docs) {
-                s_slot_start[d] = run_sl + ec;
-                if (blockIdx.x == 0) { doc_kv_start[d] = run_kv + el; doc_slot_start[d] = run_sl + ec; }
-            }
-            run_kv += tot_l;
-            run_sl += tot_c;
+    // ---- everything that is read from memory is asked for here ----
+    const int depth = mine ? slot_depth[s] : 0;
+    const int my_vis = (slot_vis && mine) ? slot_vis[s] : 0;
+    int l = t < n_docs ? doc_prefix_len[t] : 0, c = t < n_docs ? doc_branch_cnt[t] : 0;
+    uint32_t m[2] = {0u, 0u};                        // live flags of slots [64 t, 64 t + 64)
+    if ((reinterpret_cast<uintptr_t>(slot_alive) & 15) == 0 && (t + 1) * 64 <= n_slots) {
+        const uint4* v = reinterpret_cast<const uint4*>(slot_alive) + t * 4;
+        uint4 w[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) w[i] = v[i];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            m[i >> 1] |= (nonzero_bytes(w[i].x) | nonzero_bytes(w[i].y) << 4 | nonzero_bytes(w[i].z) << 8 | nonzero_bytes(w[i].w) << 12) << (16 * (i & 1));
+    } else {
+        const int n = min(max(n_slots - t * 64, 0), 64);
+#pragma unroll 8
+        for (int i = 0; i < n; ++i)
+            if (slot_alive[t * 64 + i]) m[i >> 5] |= 1u << (i & 31);
+    }
+
+    // ---- scans: live slots, and prefix tokens and slots per document (1024 documents at a time) ----
+    const int pop = __popc(m[0]) + __popc(m[1]);
+    int pop_incl = warp_incl_scan(pop);
+    int run_kv = 0, run_sl = 0, total = 0;
+    for (int base = 0; base == 0 || base < n_docs; base += kPlanThreads) {
+        if (base > 0) {
+            const int d = base + t;
+            l = d < n_docs ? doc_prefix_len[d] : 0;
+            c = d < n_docs ? doc_branch_cnt[d] : 0;
         }
-        if (threadIdx.x == 0) {
-            s_slot_start[n_docs] = run_sl;
-            if (blockIdx.x == 0) { doc_kv_start[n_docs] = run_kv; doc_slot_start[n_docs] = run_sl; }
+        if (base == 0 && lane == 31) s_cnt[warp] = pop_incl;
+        long long tot;
+        const long long ex = scan_words(words(l, c), s_scan[(base / kPlanThreads) & 1], tot);
+        const int d = base + t;
+        if (d < n_docs) {
+            const int kv0 = run_kv + word_lo(ex), sl0 = run_sl + word_hi(ex);
+            s_start[d] = sl0;
+            s_len[d] = l;
+            if (planner) { doc_kv_start[d] = kv0; doc_slot_start[d] = sl0; }
+        }
+        run_kv += word_lo(tot); run_sl += word_hi(tot);
+        if (base == 0) {
+            const int ct = s_cnt[lane];
+            const int ci = warp_incl_scan(ct);
+            const int excl = pop_incl - pop + __shfl_sync(0xffffffffu, ci - ct, warp);
+            total = __shfl_sync(0xffffffffu, ci, 31);
+            s_mask[2 * t] = m[0]; s_mask[2 * t + 1] = m[1];
+            s_pre[2 * t] = static_cast<uint16_t>(excl);               // at most 65535 wherever a live slot may follow
+            s_pre[2 * t + 1] = static_cast<uint16_t>(excl + __popc(m[0]));
         }
     }
-    // ---- live slots before this block and in total ----
-    int before, total;
-    {
-        int e0, e1, after;
-        block_excl_scan2<kFusedThreads>(count_alive(slot_alive, 0, min(first, n_slots)),
-                                        count_alive(slot_alive, min(first, n_slots), n_slots), sm2, e0, e1, before, after);
-        total = before + after;
+    if (t == 0) {
+        s_start[n_docs] = run_sl;
+        if (planner) { doc_kv_start[n_docs] = run_kv; doc_slot_start[n_docs] = run_sl; }
     }
-    int tot;
-    const int excl = before + block_excl_scan<kFusedThreads>(alive, sm, tot);
+    __syncthreads();
+    auto live_before = [&](int x) {                  // live slots below x
+        if (x >= n_slots) return total;
+        return static_cast<int>(s_pre[x >> 5]) + __popc(s_mask[x >> 5] & ((1u << (x & 31)) - 1u));
+    };
 
-    if (s < n_slots) {
-        int lo = 0, hi = n_docs;           // invariant: slot_start[lo] <= s < slot_start[hi]
+    if (!planner) {
+        if (!mine) return;
+        int lo = 0, hi = n_docs;           // invariant: start[lo] <= s < start[hi]; documents without slots share a start and are skipped
         while (hi - lo > 1) {
             const int mid = (lo + hi) >> 1;
-            if (s_slot_start[mid] <= s) lo = mid; else hi = mid;
+            if (s_start[mid] <= s) lo = mid; else hi = mid;
         }
         const int d = lo;
-        const int j = s - s_slot_start[d];
-        if (j == 0) {
-            // first slot of document d: rows before it; documents without slots just before d share the value
-            doc_active_start[d] = excl;
-            for (int e = d - 1; e >= 0 && s_slot_start[e + 1] == s_slot_start[e]; --e) doc_active_start[e] = excl;
-        }
-        if (alive) {
-            const int anchor = slot_vis ? my_vis : doc_prefix_len[d];
+        const int j = s - s_start[d];
+        const int excl = live_before(s);
+        if ((s_mask[s >> 5] >> (s & 31)) & 1u) {
+            const int anchor = slot_vis ? my_vis : (n_docs > 0 ? s_len[d] : 0);
             const int bs = anchor + j * pos_gap;
             active_slot[excl] = s;
             doc_id[excl] = d;
@@ -566,29 +582,25 @@ meta_fused_kernel(int n_docs, int n_slots, int32_t suffix_cap, int32_t pos_gap, 
             suffix_len[excl] = depth;
             if (prefix_vis) prefix_vis[excl] = anchor;
         } else {
-            const int t = total + (s - excl);            // the dead slots fill the tail of every row table with -1
-            active_slot[t] = -1; doc_id[t] = -1; branch_start[t] = -1;
-            pos_id[t] = -1; suffix_off[t] = -1; suffix_len[t] = -1;
-            if (prefix_vis) prefix_vis[t] = -1;
+            const int x = total + (s - excl);        // the dead slots fill the tail of every row table with -1
+            active_slot[x] = -1; doc_id[x] = -1; branch_start[x] = -1;
+            pos_id[x] = -1; suffix_off[x] = -1; suffix_len[x] = -1;
+            if (prefix_vis) prefix_vis[x] = -1;
         }
-    }
-    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
-        *n_active = total;
-        doc_active_start[n_docs] = total;
-        for (int e = n_docs - 1; e >= 0 && s_slot_start[e + 1] == s_slot_start[e]; --e) doc_active_start[e] = total;
+        return;
     }
 
-    // ---- the block that finishes last writes the plan ----
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) s_last = atomicAdd(&hdr->finished, 1u) == gridDim.x - 1;
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    static_assert(kFusedDocs + 1 >= kPlanScratchInts, "the document scan's shared array doubles as the plan's scratch");
-    __shared__ uint16_t s_rank[kSortItems];
-    plan_block<kFusedThreads>(n_docs, G, Hkv, n_sm, doc_prefix_len, doc_active_start, s_slot_start, s_rank,
-                              hdr, work, split, work_cap, part_cap);
+    // ---- block 0: rows per document, then the plan ----
+    for (int d = t; d <= n_docs; d += kPlanThreads) {
+        const int r = d == n_docs ? total : live_before(s_start[d]);
+        s_start[d] = r;
+        doc_active_start[d] = r;
+    }
+    if (t == 0) *n_active = total;
+    __syncthreads();                                 // the mask is not read any more: its memory serves the plan's sort
+    static_assert(kPlanScratchInts * 4 + kSortItems * 2 <= sizeof(s_bits), "the sort's keys and ranks take the mask's place");
+    plan_block(n_docs, G, Hkv, n_sm, s_len, s_start, reinterpret_cast<int*>(s_bits), reinterpret_cast<uint16_t*>(s_bits + kPlanScratchInts),
+               hdr, work, split, work_cap, part_cap);
 }
 
 // ---------------------------------------------------------------------------------------------------------------
@@ -727,12 +739,10 @@ int launch_build_meta(const hpd_geom& g, int n_docs, int n_slots, const int32_t*
     WorkItem* work = reinterpret_cast<WorkItem*>(ws + lay.off_work);
     DocSplit* split = reinterpret_cast<DocSplit*>(ws + lay.off_split);
 
-    if (n_docs <= kFusedDocs) {
-        // the header's arrival counter must read 0 at launch: plan_block leaves it so (hdr->finished = 0) after every
-        // step, and the very first step on a workspace finds whatever the caller's allocation holds -- clear it
-        HPD_CUDA_TRY(cudaMemsetAsync(&hdr->finished, 0, sizeof(hdr->finished), stream));
-        const int blocks = n_slots > 0 ? (n_slots + kFusedThreads - 1) / kFusedThreads : 1;
-        meta_fused_kernel<<<blocks, kFusedThreads, 0, stream>>>(
+    // one launch up to 4096 documents and 65536 slots: what a block can hold in shared memory (45 KB) and count in 16 bits
+    if (n_docs <= kStepDocs && n_slots <= kStepSlots) {
+        const int blocks = 1 + (n_slots + kPlanThreads - 1) / kPlanThreads;
+        meta_step_kernel<<<blocks, kPlanThreads, 0, stream>>>(
             n_docs, n_slots, g.suffix_cap, pos_gap, g.Hq / g.Hkv, g.Hkv, n_sm, doc_prefix_len, doc_branch_cnt, slot_depth,
             slot_alive, slot_vis, doc_kv_start, doc_slot_start, doc_active_start, active_slot, doc_id, branch_start, pos_id,
             suffix_off, suffix_len, prefix_vis, n_active, hdr, work, split, lay.work_cap, lay.part_cap);
