@@ -210,6 +210,11 @@ __device__ __forceinline__ float ex2(float x) {
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
+// pairs of fp32 in one 64-bit register: two fused multiply-adds or additions per instruction, each rounded as usual
+__device__ __forceinline__ uint64_t pair(float a, float b) { uint64_t r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b)); return r; }
+__device__ __forceinline__ void unpair(uint64_t v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) { uint64_t r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) { uint64_t r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
 __device__ __forceinline__ float fmax3(float a, float b, float c) {
     float d;
     asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
@@ -688,26 +693,30 @@ hpd_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             const bool row_valid = row < nrows;
             const bool warp_active = quad * 32 < nrows;
             float m = -INFINITY, l = 0.f;
+            // tiles [j_pre, j_full): prefix tiles that every row of the warp sees whole, no window to compute and nothing to mask
+            const int nbt = BLOCK ? block_tiles(u) : 0;
+            const int ns = nt - u.np - nbt, j_pre = ns + nbt;
+            const int my_keys = ORDER && row_valid ? min(u.key_count, my_pv) : u.key_count;
+            const int j_full = j_pre + (ORDER ? __reduce_min_sync(0xffffffffu, max(my_keys, 0)) : u.key_count) / kN;
             for (int j = 0; j < nt && ok; ++j) {
                 // Columns of this tile the row may see.  A suffix tile holds a few branches each; a warp whose rows see
                 // none of them (known from the descriptor alone) skips the tile's scores and writes zero probabilities.
-                int lo = 0, hi = 0;
-                if (warp_active) {
-                    const int nbt = BLOCK ? block_tiles(u) : 0;
-                    const int ns = nt - u.np - nbt;
-                    if (BLOCK && j >= ns && j < ns + nbt) {
+                int lo = 0, hi = kN;
+                bool vis = warp_active, whole = true;
+                if (warp_active && (j < j_pre || j >= j_full)) {
+                    if (BLOCK && j >= ns && j < j_pre) {
                         hi = min(kN, u.blk_count - (j - ns) * kN);
-                    } else if (j >= ns) {
-                        hi = min(kN, (ORDER ? min(u.key_count, my_pv) : u.key_count) - (j - ns - nbt) * kN);
-                        if (hi < 0) hi = 0;
+                    } else if (j >= j_pre) {
+                        hi = max(0, min(kN, my_keys - (j - j_pre) * kN));
                     } else {
                         const int base = j * kN;
                         lo = max(0, my_cs - base);
                         hi = min(kN, my_cs + my_len - base);
                         if (hi < lo) hi = lo;
                     }
+                    vis = __any_sync(0xffffffffu, hi > lo);
+                    whole = __all_sync(0xffffffffu, lo == 0 && hi == kN);
                 }
-                const bool vis = __any_sync(0xffffffffu, hi > lo);
                 const int pb = pw & 1;                   // the tile's S / P buffer
                 const uint32_t tmem_s = tmem_s0 + pb * kN;
                 ok = mbar_wait_warp(&misc->s_full[x][pb], (pw >> 1) & 1, misc);
@@ -720,7 +729,7 @@ hpd_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 }
 
                 if (vis) {
-                    if (!__all_sync(0xffffffffu, lo == 0 && hi == kN)) {
+                    if (!whole) {
                         const unsigned span = static_cast<unsigned>(hi - lo);
 #pragma unroll
                         for (int c = 0; c < kN; ++c)
@@ -748,7 +757,7 @@ hpd_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                                 tc_fence_after();
                                 const float m_new = grow ? tmax : m;
                                 const float f = grow ? ex2(m - m_new) : 1.f;
-#pragma unroll
+#pragma unroll 1
                                 for (int c0 = 0; c0 < D; c0 += 32) {
                                     uint32_t ov[32];
                                     tmem_ld32(tmem_o + c0, ov);
@@ -777,20 +786,25 @@ hpd_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                         tmem_st16(tmem_s + 16, pk);
                     } else {
                         const float neg_m = (m == -INFINITY) ? 0.f : -m;
-                        float lsum[4] = {0.f, 0.f, 0.f, 0.f};
+                        const uint64_t sc2 = pair(p.scale_log2, p.scale_log2), nm2 = pair(neg_m, neg_m);
+                        uint64_t ls0 = pair(0.f, 0.f), ls1 = ls0;
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {    // 32 keys = 16 columns of bf16 pairs per store
                             uint32_t pk[16];
 #pragma unroll
                             for (int c = 0; c < 16; ++c) {
-                                const float e0 = ex2(fmaf(__uint_as_float(sv[h * 32 + 2 * c]), p.scale_log2, neg_m));
-                                const float e1 = ex2(fmaf(__uint_as_float(sv[h * 32 + 2 * c + 1]), p.scale_log2, neg_m));
-                                lsum[c & 1] += e0; lsum[2 + (c & 1)] += e1;
+                                const uint64_t y = fma2(pair(__uint_as_float(sv[h * 32 + 2 * c]), __uint_as_float(sv[h * 32 + 2 * c + 1])), sc2, nm2);
+                                float y0, y1;
+                                unpair(y, y0, y1);
+                                const float e0 = ex2(y0), e1 = ex2(y1);
+                                if (c & 1) ls1 = add2(ls1, pair(e0, e1)); else ls0 = add2(ls0, pair(e0, e1));
                                 pk[c] = pack_bf16(e0, e1);
                             }
                             tmem_st16(tmem_s + h * 16, pk);
                         }
-                        l += (lsum[0] + lsum[1]) + (lsum[2] + lsum[3]);
+                        float a0, a1;
+                        unpair(add2(ls0, ls1), a0, a1);
+                        l += a0 + a1;
                     }
                     tmem_st_wait();
                 }
@@ -816,24 +830,30 @@ hpd_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             const float inv = final_out ? (l > 0.f ? 1.f / l : 0.f) : 1.f;
             const int64_t pr = (static_cast<int64_t>(final_out ? 0 : u.part_base) + u.row_begin + b_row) * p.a.g.Hq + hq;
             float* po = p.part_o + pr * D;
-#pragma unroll
-            for (int c0 = 0; c0 < D; c0 += 32) {
-                float acc[32];
-#pragma unroll
-                for (int c = 0; c < 32; ++c) acc[c] = 0.f;
+            // the accumulator, 32 columns at a time; rolled: the code of the epilogue runs once per unit, out of a cold instruction
+            // cache (unrolled, four times as long, it took the 64-prompt step from 183 to 186 us, the shared block's from 175 to 182)
+            auto read_o = [&](int c0, float (&acc)[32]) {
                 if (warp_active && nt > 0) {
                     uint32_t ov[32];
                     tmem_ld32(tmem_o + c0, ov);
                     tmem_ld_wait();
 #pragma unroll
                     for (int c = 0; c < 32; ++c) acc[c] = inv * __uint_as_float(ov[c]);
+                } else {
+#pragma unroll
+                    for (int c = 0; c < 32; ++c) acc[c] = 0.f;
                 }
                 if (c0 + 32 >= D) {                      // all TMEM reads of this unit are done
                     tc_fence_before();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&misc->o_free[x]);
                 }
-                if (final_out) {
+            };
+            if (final_out) {
+#pragma unroll 1
+                for (int c0 = 0; c0 < D; c0 += 32) {
+                    float acc[32];
+                    read_o(c0, acc);
                     // transpose through this warp's 2 KB of shared memory: a row's 32 columns go out as one 64-byte
                     // piece, 8 rows per store instruction
 #pragma unroll
@@ -857,10 +877,17 @@ hpd_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                             *reinterpret_cast<uint4*>(p.a.o + (static_cast<int64_t>(grow) * p.a.g.Hq + u.head * G + tg) * D + c0 + ch * 8) = pk;
                     }
                     __syncwarp();
-                } else if (store) {
+                }
+            } else {
+#pragma unroll 1
+                for (int c0 = 0; c0 < D; c0 += 32) {
+                    float acc[32];
+                    read_o(c0, acc);
+                    if (store) {
 #pragma unroll
-                    for (int c = 0; c < 32; c += 4)
-                        *reinterpret_cast<float4*>(po + c0 + c) = make_float4(acc[c], acc[c + 1], acc[c + 2], acc[c + 3]);
+                        for (int c = 0; c < 32; c += 4)
+                            *reinterpret_cast<float4*>(po + c0 + c) = make_float4(acc[c], acc[c + 1], acc[c + 2], acc[c + 3]);
+                    }
                 }
             }
             if (store) {
