@@ -663,7 +663,7 @@ prefill_meta_kernel(int n_docs, int G, int32_t pos_gap,
     }
     for (int x = blockIdx.x * kPrefillThreads + threadIdx.x; x < n_items; x += stride) {
         const int d = doc_of(s_item, x);
-        const int m = x - s_item[d];
+        const int m = s_item[d + 1] - 1 - x;         // a prompt's last block has the most keys: longest first (step of 1 prompt 81 -> 71 us)
         const int L = s_kv[d + 1] - s_kv[d];
         WorkItem it;
         it.doc = d; it.key_begin = 0; it.key_count = min(L, (m + 1) * rpb);
@@ -680,7 +680,7 @@ prefill_meta_kernel(int n_docs, int G, int32_t pos_gap,
         if (threadIdx.x == 0) {
             *n_tokens = n_tok;
             hdr->n_work = n_items; hdr->chunk_tokens = 0; hdr->n_part_rows = 0; hdr->any_split = 0;
-            hdr->ticket = 0; hdr->finished = 0; hdr->work_cap = work_cap; hdr->part_cap = part_cap; hdr->longest_first = 0;
+            hdr->ticket = 0; hdr->finished = 0; hdr->work_cap = work_cap; hdr->part_cap = part_cap; hdr->longest_first = n_docs == 1;
         }
     }
 }
