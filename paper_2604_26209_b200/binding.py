@@ -2,8 +2,9 @@
 
 Argument marshalling only: tensors are passed as raw device pointers together with the current
 CUDA stream; every step of the path runs in the library's kernels.  PyTorch is used for device
-memory and streams.  The library must be present -- there is no fallback; ``load()`` raises if
-``libhpd.so`` has not been built (``python -m paper_2604_26209_b200.build``).
+memory and streams.  The calls of a step go through ``_host.so`` (native marshalling, ``csrc/host.cpp``: ctypes took longer
+than the GPU for a small step), the others through ctypes.  Both libraries must be present -- there is no fallback;
+``load()`` raises if they have not been built (``python -m paper_2604_26209_b200.build``).
 """
 from __future__ import annotations
 
@@ -34,10 +35,11 @@ class HpdError(RuntimeError):
 
 
 _lib = None
+_host = None
 
 
 def load() -> C.CDLL:
-    global _lib
+    global _lib, _host
     if _lib is None:
         if not os.path.exists(LIB_PATH):
             raise HpdError(f"{LIB_PATH} is missing: build it with `python -m paper_2604_26209_b200.build` "
@@ -87,8 +89,21 @@ def load() -> C.CDLL:
         lib.std_attn_decode_static_max_bytes.argtypes = []
         lib.std_attn_decode_static.restype = C.c_int
         lib.std_attn_decode_static.argtypes = [C.POINTER(HpdGeom), C.c_int, C.c_int, C.c_longlong] + [vp] * 8 + [vp]
+        try:
+            from . import _host as host
+        except ImportError as e:
+            raise HpdError(f"_host.so is missing or does not fit this interpreter: build it with `python -m "
+                           f"paper_2604_26209_b200.build` ({e})") from e
+        for name in host.ENTRIES:
+            host.set_address(name, C.cast(getattr(lib, name), C.c_void_p).value)
+        _host = host
         _lib = lib
     return _lib
+
+
+def _calls():
+    """The native entry points (arguments of the C function in order, without the stream)."""
+    return _host if _lib is not None else (load(), _host)[1]
 
 
 def make_geom(g) -> HpdGeom:
@@ -155,36 +170,33 @@ class MetaTables:
 
 
 def hpd_build_meta(geom, n_docs, n_slots, doc_prefix_len, doc_branch_cnt, slot_depth, slot_alive, pos_gap, m: MetaTables):
-    g = make_geom(geom)
-    rc = load().hpd_build_meta(C.byref(g), n_docs, n_slots, _ptr(doc_prefix_len), _ptr(doc_branch_cnt), _ptr(slot_depth),
-                               _ptr(slot_alive), int(pos_gap), _ptr(m.doc_kv_start), _ptr(m.doc_slot_start),
-                               _ptr(m.doc_active_start), _ptr(m.active_slot), _ptr(m.doc_id), _ptr(m.branch_start),
-                               _ptr(m.pos_id), _ptr(m.suffix_off), _ptr(m.suffix_len), _ptr(m.n_active),
-                               _ptr(m.workspace), m.workspace.numel(), _ptr(m.dev_status), _stream())
+    rc = _calls().hpd_build_meta(geom, n_docs, n_slots, doc_prefix_len, doc_branch_cnt, slot_depth,
+                                 slot_alive, int(pos_gap), m.doc_kv_start, m.doc_slot_start,
+                                 m.doc_active_start, m.active_slot, m.doc_id, m.branch_start,
+                                 m.pos_id, m.suffix_off, m.suffix_len, m.n_active,
+                                 m.workspace, m.workspace.numel(), m.dev_status)
     _check(rc, "hpd_build_meta")
 
 
 def hpd_build_meta_skeleton(geom, n_docs, n_slots, doc_prefix_len, doc_branch_cnt, slot_depth, slot_alive, slot_vis, pos_gap,
                             m: MetaTables):
-    g = make_geom(geom)
-    rc = load().hpd_build_meta_skeleton(C.byref(g), n_docs, n_slots, _ptr(doc_prefix_len), _ptr(doc_branch_cnt),
-                                        _ptr(slot_depth), _ptr(slot_alive), _ptr(slot_vis), int(pos_gap),
-                                        _ptr(m.doc_kv_start), _ptr(m.doc_slot_start), _ptr(m.doc_active_start),
-                                        _ptr(m.active_slot), _ptr(m.doc_id), _ptr(m.branch_start), _ptr(m.pos_id),
-                                        _ptr(m.suffix_off), _ptr(m.suffix_len), _ptr(m.prefix_vis), _ptr(m.n_active),
-                                        _ptr(m.workspace), m.workspace.numel(), _ptr(m.dev_status), _stream())
+    rc = _calls().hpd_build_meta_skeleton(geom, n_docs, n_slots, doc_prefix_len, doc_branch_cnt,
+                                          slot_depth, slot_alive, slot_vis, int(pos_gap),
+                                          m.doc_kv_start, m.doc_slot_start, m.doc_active_start,
+                                          m.active_slot, m.doc_id, m.branch_start, m.pos_id,
+                                          m.suffix_off, m.suffix_len, m.prefix_vis, m.n_active,
+                                          m.workspace, m.workspace.numel(), m.dev_status)
     _check(rc, "hpd_build_meta_skeleton")
 
 
 def hpd_attn_decode_posorder(geom, n_docs, max_rows, n_slots, total_prefix_tokens, q, prefix_k, prefix_v, suffix_k, suffix_v,
                              doc_prefix_len, slot_depth, slot_alive, m: MetaTables, suffix_includes_new, o, lse=None):
-    g = make_geom(geom)
-    rc = load().hpd_attn_decode_posorder(C.byref(g), n_docs, max_rows, n_slots, total_prefix_tokens, _ptr(q), _ptr(prefix_k),
-                                         _ptr(prefix_v), _ptr(suffix_k), _ptr(suffix_v), _ptr(m.doc_kv_start),
-                                         _ptr(doc_prefix_len), _ptr(m.doc_active_start), _ptr(m.doc_slot_start),
-                                         _ptr(m.doc_id), _ptr(m.active_slot), _ptr(slot_depth), _ptr(slot_alive),
-                                         _ptr(m.prefix_vis), _ptr(m.n_active), int(bool(suffix_includes_new)), _ptr(o),
-                                         _ptr(lse), _ptr(m.workspace), m.workspace.numel(), _ptr(m.dev_status), _stream())
+    rc = _calls().hpd_attn_decode_posorder(geom, n_docs, max_rows, n_slots, total_prefix_tokens, q, prefix_k,
+                                           prefix_v, suffix_k, suffix_v, m.doc_kv_start,
+                                           doc_prefix_len, m.doc_active_start, m.doc_slot_start,
+                                           m.doc_id, m.active_slot, slot_depth, slot_alive,
+                                           m.prefix_vis, m.n_active, int(bool(suffix_includes_new)), o,
+                                           lse, m.workspace, m.workspace.numel(), m.dev_status)
     _check(rc, "hpd_attn_decode_posorder")
 
 
@@ -209,78 +221,68 @@ class PrefillTables:
 
 
 def hpd_prefill_meta(geom, n_docs, n_slots, total_tokens, doc_prefix_len, doc_branch_cnt, slot_vis, pos_gap, t: PrefillTables):
-    g = make_geom(geom)
-    rc = load().hpd_prefill_meta(C.byref(g), n_docs, n_slots, total_tokens, _ptr(doc_prefix_len), _ptr(doc_branch_cnt),
-                                 _ptr(slot_vis), int(pos_gap), _ptr(t.doc_kv_start), _ptr(t.doc_slot_start), _ptr(t.tok_doc),
-                                 _ptr(t.tok_pos), _ptr(t.tok_vis), _ptr(t.n_tokens), _ptr(t.workspace), t.workspace.numel(),
-                                 _stream())
+    rc = _calls().hpd_prefill_meta(geom, n_docs, n_slots, total_tokens, doc_prefix_len, doc_branch_cnt,
+                                   slot_vis, int(pos_gap), t.doc_kv_start, t.doc_slot_start, t.tok_doc,
+                                   t.tok_pos, t.tok_vis, t.n_tokens, t.workspace, t.workspace.numel())
     _check(rc, "hpd_prefill_meta")
 
 
 def hpd_prefill_attn(geom, n_docs, total_tokens, q, prefix_k, prefix_v, doc_prefix_len, t: PrefillTables, o, lse=None):
-    g = make_geom(geom)
-    rc = load().hpd_prefill_attn(C.byref(g), n_docs, total_tokens, _ptr(q), _ptr(prefix_k), _ptr(prefix_v),
-                                 _ptr(t.doc_kv_start), _ptr(doc_prefix_len), _ptr(t.tok_doc), _ptr(t.tok_vis), _ptr(t.n_tokens),
-                                 _ptr(o), _ptr(lse), _ptr(t.workspace), t.workspace.numel(), _ptr(t.dev_status), _stream())
+    rc = _calls().hpd_prefill_attn(geom, n_docs, total_tokens, q, prefix_k, prefix_v,
+                                   t.doc_kv_start, doc_prefix_len, t.tok_doc, t.tok_vis, t.n_tokens,
+                                   o, lse, t.workspace, t.workspace.numel(), t.dev_status)
     _check(rc, "hpd_prefill_attn")
 
 
 def hpd_attn_decode_shared(geom, n_docs, max_rows, n_slots, total_prefix_tokens, q, prefix_k, prefix_v, suffix_k, suffix_v,
                            block_k, block_v, total_block_tokens, doc_block, block_kv_start, block_len,
                            doc_prefix_len, m: MetaTables, suffix_includes_new, o, lse=None):
-    g = make_geom(geom)
-    rc = load().hpd_attn_decode_shared(C.byref(g), n_docs, max_rows, n_slots, total_prefix_tokens, _ptr(q), _ptr(prefix_k),
-                                       _ptr(prefix_v), _ptr(suffix_k), _ptr(suffix_v), _ptr(block_k), _ptr(block_v),
-                                       int(total_block_tokens), _ptr(doc_block), _ptr(block_kv_start), _ptr(block_len),
-                                       _ptr(m.doc_kv_start), _ptr(doc_prefix_len), _ptr(m.doc_active_start), _ptr(m.doc_id),
-                                       _ptr(m.suffix_off), _ptr(m.suffix_len), _ptr(m.n_active), int(bool(suffix_includes_new)),
-                                       _ptr(o), _ptr(lse), _ptr(m.workspace), m.workspace.numel(), _ptr(m.dev_status), _stream())
+    rc = _calls().hpd_attn_decode_shared(geom, n_docs, max_rows, n_slots, total_prefix_tokens, q, prefix_k,
+                                         prefix_v, suffix_k, suffix_v, block_k, block_v,
+                                         int(total_block_tokens), doc_block, block_kv_start, block_len,
+                                         m.doc_kv_start, doc_prefix_len, m.doc_active_start, m.doc_id,
+                                         m.suffix_off, m.suffix_len, m.n_active, int(bool(suffix_includes_new)),
+                                         o, lse, m.workspace, m.workspace.numel(), m.dev_status)
     _check(rc, "hpd_attn_decode_shared")
 
 
 def hpd_merge_lse(geom, max_rows, n_active, o_a, lse_a, o_b, lse_b, o, lse=None):
-    g = make_geom(geom)
-    rc = load().hpd_merge_lse(C.byref(g), max_rows, _ptr(n_active), _ptr(o_a), _ptr(lse_a), _ptr(o_b), _ptr(lse_b), _ptr(o),
-                              _ptr(lse), _stream())
+    rc = _calls().hpd_merge_lse(geom, max_rows, n_active, o_a, lse_a, o_b, lse_b, o,
+                                lse)
     _check(rc, "hpd_merge_lse")
 
 
 def hpd_advance(geom, max_rows, n_active, active_slot, token_id, delimiter_id, slot_depth, slot_alive, n_alive):
-    g = make_geom(geom)
-    rc = load().hpd_advance(C.byref(g), max_rows, _ptr(n_active), _ptr(active_slot), _ptr(token_id), int(delimiter_id),
-                            _ptr(slot_depth), _ptr(slot_alive), _ptr(n_alive), _stream())
+    rc = _calls().hpd_advance(geom, max_rows, n_active, active_slot, token_id, int(delimiter_id),
+                              slot_depth, slot_alive, n_alive)
     _check(rc, "hpd_advance")
 
 
 def hpd_rope(geom, max_rows, n_active, pos_id, q, k_new):
-    g = make_geom(geom)
-    _check(load().hpd_rope(C.byref(g), max_rows, _ptr(n_active), _ptr(pos_id), _ptr(q), _ptr(k_new), _stream()), "hpd_rope")
+    _check(_calls().hpd_rope(geom, max_rows, n_active, pos_id, q, k_new), "hpd_rope")
 
 
 def hpd_kv_append(geom, max_rows, n_slots, n_active, suffix_off, suffix_len, k_new, v_new, suffix_k, suffix_v, dev_status):
-    g = make_geom(geom)
-    rc = load().hpd_kv_append(C.byref(g), max_rows, n_slots, _ptr(n_active), _ptr(suffix_off), _ptr(suffix_len),
-                              _ptr(k_new), _ptr(v_new), _ptr(suffix_k), _ptr(suffix_v), _ptr(dev_status), _stream())
+    rc = _calls().hpd_kv_append(geom, max_rows, n_slots, n_active, suffix_off, suffix_len,
+                                k_new, v_new, suffix_k, suffix_v, dev_status)
     _check(rc, "hpd_kv_append")
 
 
 def hpd_rope_append(geom, max_rows, n_slots, n_active, pos_id, suffix_off, suffix_len, q, k_new, v_new, suffix_k, suffix_v,
                     dev_status):
-    g = make_geom(geom)
-    rc = load().hpd_rope_append(C.byref(g), max_rows, n_slots, _ptr(n_active), _ptr(pos_id), _ptr(suffix_off),
-                                _ptr(suffix_len), _ptr(q), _ptr(k_new), _ptr(v_new), _ptr(suffix_k), _ptr(suffix_v),
-                                _ptr(dev_status), _stream())
+    rc = _calls().hpd_rope_append(geom, max_rows, n_slots, n_active, pos_id, suffix_off,
+                                  suffix_len, q, k_new, v_new, suffix_k, suffix_v,
+                                  dev_status)
     _check(rc, "hpd_rope_append")
 
 
 def hpd_attn_decode(geom, n_docs, max_rows, n_slots, total_prefix_tokens, q, prefix_k, prefix_v, suffix_k, suffix_v,
                     doc_prefix_len, m: MetaTables, suffix_includes_new, o, lse=None):
-    g = make_geom(geom)
-    rc = load().hpd_attn_decode(C.byref(g), n_docs, max_rows, n_slots, total_prefix_tokens, _ptr(q), _ptr(prefix_k),
-                                _ptr(prefix_v), _ptr(suffix_k), _ptr(suffix_v), _ptr(m.doc_kv_start),
-                                _ptr(doc_prefix_len), _ptr(m.doc_active_start), _ptr(m.doc_id), _ptr(m.suffix_off),
-                                _ptr(m.suffix_len), _ptr(m.n_active), int(bool(suffix_includes_new)), _ptr(o), _ptr(lse),
-                                _ptr(m.workspace), m.workspace.numel(), _ptr(m.dev_status), _stream())
+    rc = _calls().hpd_attn_decode(geom, n_docs, max_rows, n_slots, total_prefix_tokens, q, prefix_k,
+                                  prefix_v, suffix_k, suffix_v, m.doc_kv_start,
+                                  doc_prefix_len, m.doc_active_start, m.doc_id, m.suffix_off,
+                                  m.suffix_len, m.n_active, int(bool(suffix_includes_new)), o, lse,
+                                  m.workspace, m.workspace.numel(), m.dev_status)
     _check(rc, "hpd_attn_decode")
 
 

@@ -1,4 +1,5 @@
-"""Compile the CUDA sources in-tree into ``libhpd.so`` for sm_100a (``python -m paper_2604_26209_b200.build``)."""
+"""Compile the CUDA sources in-tree into ``libhpd.so`` for sm_100a and the Python side of its calls into ``_host.so``
+(``python -m paper_2604_26209_b200.build``)."""
 from __future__ import annotations
 
 import concurrent.futures as cf
@@ -6,11 +7,13 @@ import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libhpd.so")
+HOST = os.path.join(HERE, "_host.so")
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std=c++17",
               "-Xcompiler", "-fPIC", "-Xcompiler", "-Wall", "-Xptxas", "-v"]
@@ -43,14 +46,38 @@ def _compile(src: str, verbose: bool) -> str:
     return obj
 
 
+def _build_host() -> None:
+    src = os.path.join(CSRC, "host.cpp")
+    if os.path.exists(HOST) and os.path.getmtime(HOST) >= max(os.path.getmtime(src), _deps_mtime()):
+        return
+    import torch
+    root = os.path.dirname(torch.__file__)
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    inc = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
+           os.path.join(cuda, "include"), sysconfig.get_paths()["include"]]
+    tmp = HOST + f".tmp{os.getpid()}"
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-Wall", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           *["-isystem" + i for i in inc], src, "-o", tmp, "-L" + os.path.join(root, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu",
+           "-ltorch_python"]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        sys.stderr.write(res.stdout + res.stderr)
+        raise RuntimeError(f"g++ failed on {src}")
+    os.replace(tmp, HOST)
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(OBJ, exist_ok=True)
     srcs = sorted(glob.glob(os.path.join(CSRC, "*.cu")))
     if force:
         for f in glob.glob(os.path.join(OBJ, "*.o")):
             os.remove(f)
-    with cf.ThreadPoolExecutor(max_workers=min(8, len(srcs))) as ex:
+        if os.path.exists(HOST):
+            os.remove(HOST)
+    with cf.ThreadPoolExecutor(max_workers=min(8, len(srcs)) + 1) as ex:
+        host = ex.submit(_build_host)
         objs = list(ex.map(lambda s: _compile(s, verbose), srcs))
+        host.result()
     if (not os.path.exists(LIB)) or any(os.path.getmtime(o) > os.path.getmtime(LIB) for o in objs):
         tmp = LIB + f".tmp{os.getpid()}"
         subprocess.run([_nvcc(), "-shared", "-o", tmp, *objs, "-gencode", "arch=compute_100a,code=sm_100a"], check=True)

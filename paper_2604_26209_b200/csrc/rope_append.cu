@@ -204,10 +204,16 @@ kv_append_kernel(int row_u4 /* Hkv*D*2/16 */, int32_t suffix_cap, int64_t cache_
     }
 }
 
-InvFreq inv_freq_table(const hpd_geom& g)
+// Each thread keeps the table of its last (theta, D): a model asks for the same one layer after layer, and 64 powers take 3 us.
+const InvFreq& inv_freq_table(const hpd_geom& g)
 {
-    InvFreq t{};
-    for (int i = 0; i < g.D / 2; ++i) t.f[i] = pow(static_cast<double>(g.rope_theta), -2.0 * i / static_cast<double>(g.D));
+    static thread_local InvFreq t;
+    static thread_local float theta = -1.f;
+    static thread_local int dim = 0;
+    if (g.rope_theta != theta || g.D != dim) {
+        for (int i = 0; i < g.D / 2; ++i) t.f[i] = pow(static_cast<double>(g.rope_theta), -2.0 * i / static_cast<double>(g.D));
+        theta = g.rope_theta; dim = g.D;
+    }
     return t;
 }
 
@@ -296,7 +302,7 @@ int launch_rope(const hpd_geom& g, int max_rows, const int32_t* n_active, const 
                 __nv_bfloat16* q, __nv_bfloat16* k_new, cudaStream_t stream)
 {
     if (max_rows <= 0) return HPD_OK;
-    const InvFreq c = inv_freq_table(g);
+    const InvFreq& c = inv_freq_table(g);
     const AppendDst none{};
     if (g.D == 128)
         rope_kernel<128, false><<<(max_rows + kRopeRows - 1) / kRopeRows, kRopeThreads, 0, stream>>>(g.Hq, g.Hkv, c, n_active, pos_id, q, k_new, none);
@@ -312,7 +318,7 @@ int launch_rope_append(const hpd_geom& g, int max_rows, int n_slots, const int32
                        cudaStream_t stream)
 {
     if (max_rows <= 0) return HPD_OK;
-    const InvFreq c = inv_freq_table(g);
+    const InvFreq& c = inv_freq_table(g);
     const AppendDst ad{g.suffix_cap, static_cast<int64_t>(n_slots) * g.suffix_cap, suffix_off, suffix_len, v_new,
                        suffix_k, suffix_v, dev_status};
     if (g.D == 128)
