@@ -354,6 +354,8 @@ hpd_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(&misc->tmem_base);
+    start_dependents();
+    await_predecessors();                                // nothing in global memory has been touched so far
 
     if (warp == 0 || warp == 3) {
         // ============================ scheduler and TMA producer of one pipeline =====================
@@ -929,6 +931,8 @@ template <int D>
 __global__ void __launch_bounds__(256)
 hpd_merge_kernel(TcParams p, const DocSplit* __restrict__ split)
 {
+    start_dependents();
+    await_predecessors();
     // the attention kernel drew its units from the ticket counter: rewind it for the next launch on this workspace
     if (blockIdx.x == 0 && threadIdx.x == 0) const_cast<WsHeader*>(p.hdr)->ticket = 0;
     if (!p.hdr->any_split) return;
@@ -1097,14 +1101,13 @@ int launch_d(const AttnArgs& a)
             return HPD_E_CUDA;
         }
     }
-    hpd_attn_tc_kernel<D, ORDER, BLOCK><<<n_sm, kThreads, C::SMEM, a.stream>>>(mq, mk, mv, mbk, mbv, sm, p);
+    HPD_CUDA_TRY(launch_chained(hpd_attn_tc_kernel<D, ORDER, BLOCK>, n_sm, kThreads, C::SMEM, a.stream, mq, mk, mv, mbk, mbv, sm, p));
     // one warp per (row, q head) where the rows allow it, at most one resident wave; with many documents nothing is
     // split as a rule (the kernel then only rewinds the ticket counter) and a small grid is launched sooner
     const long long merge_blocks = (static_cast<long long>(a.max_rows) * a.g.Hq + 7) / 8;
     const long long merge_cap = static_cast<long long>(a.n_docs) * a.g.Hkv < 4ll * n_sm ? 8ll * n_sm : 2ll * n_sm;
     const int merge_grid = static_cast<int>(std::min<long long>(std::max<long long>(merge_blocks, 1), merge_cap));
-    hpd_merge_kernel<D><<<merge_grid, 256, 0, a.stream>>>(p, reinterpret_cast<const DocSplit*>(ws + a.lay.off_split));
-    HPD_CUDA_TRY(cudaGetLastError());
+    HPD_CUDA_TRY(launch_chained(hpd_merge_kernel<D>, merge_grid, 256, 0, a.stream, p, reinterpret_cast<const DocSplit*>(ws + a.lay.off_split)));
     return HPD_OK;
 }
 

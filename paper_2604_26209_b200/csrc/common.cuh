@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <utility>
+
 #include "../../include/hpd.h"
 
 namespace hpd {
@@ -150,6 +152,28 @@ int launch_merge_lse(const hpd_geom& g, int max_rows, const int32_t* n_active, c
                      const __nv_bfloat16* o_b, const float* lse_b, __nv_bfloat16* o, float* lse, cudaStream_t stream);
 int launch_attn_std(const StdArgs& a);         // TMA ring + warp-level tensor-core instructions
 int launch_attn_tc(const AttnArgs& a);       // tcgen05 / TMA kernel
+
+// ---------------------------------------------------------------------------------------------
+// Launches that may start while their predecessor in the stream ends.  The kernel is scheduled as soon as every block of the
+// predecessor has called start_dependents() (or has ended), does what needs no memory of others, and calls
+// await_predecessors() before its first access to global memory; that returns once the predecessor has completed and its
+// writes are visible.  Every kernel launched like this waits in all of its blocks, so "the predecessor has completed"
+// includes everything before it.
+// ---------------------------------------------------------------------------------------------
+__device__ __forceinline__ void await_predecessors() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void start_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... P, typename... A>
+cudaError_t launch_chained(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t stream, A&&... args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid); cfg.blockDim = dim3(block); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
 
 // ---------------------------------------------------------------------------------------------
 // small device helpers

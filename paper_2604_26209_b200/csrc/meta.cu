@@ -500,6 +500,8 @@ meta_step_kernel(int n_docs, int n_slots, int32_t suffix_cap, int32_t pos_gap, i
     const int s = (static_cast<int>(blockIdx.x) - 1) * kPlanThreads + t;
     const bool mine = !planner && s < n_slots;
 
+    start_dependents();
+    await_predecessors();
     // ---- everything that is read from memory is asked for here ----
     const int depth = mine ? slot_depth[s] : 0;
     const int my_vis = (slot_vis && mine) ? slot_vis[s] : 0;
@@ -624,6 +626,8 @@ prefill_meta_kernel(int n_docs, int G, int32_t pos_gap,
     __shared__ int sm[kPrefillThreads / 32 + 1];
     __shared__ int s_kv[kPrefillDocs + 1], s_slot[kPrefillDocs + 1], s_item[kPrefillDocs + 1];
     const int rpb = kTileM / G;                      // tokens per row block
+    start_dependents();
+    await_predecessors();
     int run_kv = 0, run_sl = 0, run_it = 0;
     for (int base = 0; base < n_docs; base += kPrefillThreads) {
         const int d = base + threadIdx.x;
@@ -697,11 +701,10 @@ int launch_prefill_meta(const hpd_geom& g, int n_docs, int total_tokens, int32_t
     int blocks = (total_tokens + kPrefillThreads - 1) / kPrefillThreads;
     if (blocks < 1) blocks = 1;
     if (blocks > 4 * n_sm) blocks = 4 * n_sm;
-    prefill_meta_kernel<<<blocks, kPrefillThreads, 0, stream>>>(
+    HPD_CUDA_TRY(launch_chained(prefill_meta_kernel, blocks, kPrefillThreads, 0, stream,
         n_docs, g.Hq / g.Hkv, pos_gap, doc_prefix_len, doc_branch_cnt, slot_vis, doc_kv_start, doc_slot_start, tok_doc, tok_pos,
         tok_vis, n_tokens, reinterpret_cast<WsHeader*>(ws), reinterpret_cast<WorkItem*>(ws + lay.off_work),
-        reinterpret_cast<DocSplit*>(ws + lay.off_split), lay.work_cap, lay.part_cap);
-    HPD_CUDA_TRY(cudaGetLastError());
+        reinterpret_cast<DocSplit*>(ws + lay.off_split), lay.work_cap, lay.part_cap));
     return HPD_OK;
 }
 
@@ -742,11 +745,10 @@ int launch_build_meta(const hpd_geom& g, int n_docs, int n_slots, const int32_t*
     // one launch up to 4096 documents and 65536 slots: what a block can hold in shared memory (45 KB) and count in 16 bits
     if (n_docs <= kStepDocs && n_slots <= kStepSlots) {
         const int blocks = 1 + (n_slots + kPlanThreads - 1) / kPlanThreads;
-        meta_step_kernel<<<blocks, kPlanThreads, 0, stream>>>(
+        HPD_CUDA_TRY(launch_chained(meta_step_kernel, blocks, kPlanThreads, 0, stream,
             n_docs, n_slots, g.suffix_cap, pos_gap, g.Hq / g.Hkv, g.Hkv, n_sm, doc_prefix_len, doc_branch_cnt, slot_depth,
             slot_alive, slot_vis, doc_kv_start, doc_slot_start, doc_active_start, active_slot, doc_id, branch_start, pos_id,
-            suffix_off, suffix_len, prefix_vis, n_active, hdr, work, split, lay.work_cap, lay.part_cap);
-        HPD_CUDA_TRY(cudaGetLastError());
+            suffix_off, suffix_len, prefix_vis, n_active, hdr, work, split, lay.work_cap, lay.part_cap));
         return HPD_OK;
     }
     doc_scan_kernel<<<1, kScanThreads, 0, stream>>>(n_docs, doc_prefix_len, doc_branch_cnt, doc_kv_start, doc_slot_start);
