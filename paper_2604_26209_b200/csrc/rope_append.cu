@@ -1,6 +1,6 @@
 // hpd_rope, hpd_kv_append and their fusion hpd_rope_append: the streaming kernels around the attention.
 //
-// All are pure HBM streaming (read + write of the step's new q/k/v rows); one CTA per four rows (rotation) or per
+// All are pure HBM streaming (read + write of the step's new q/k/v rows); one CTA per two rows (rotation) or per
 // row (append), 16-byte accesses, grid sized by max_rows with an early exit on the device-side row count.
 // The fused kernel rotates q and k in place, and while a rotated key chunk is still in registers also
 // stores it to the row's slot in the branch cache, then copies the value row there: one launch and one
@@ -11,11 +11,16 @@ namespace hpd {
 
 namespace {
 
-constexpr int kRopeThreads = 256;
-constexpr unsigned kOneWave = 4 * 148;               // CTAs that are resident at once on any B200
-constexpr int kRopeRows = 4;                         // rows per CTA: 4 x 64 angles give every thread one to evaluate
+constexpr int kRopeThreads = 128;
+constexpr unsigned kOneWave = 6 * 148;               // CTAs of the fused kernel that are resident at once (80 registers x 128 threads)
+constexpr int kRopeRows = 2;                         // rows per CTA: 2 x 64 angles give every thread one to evaluate
 
-// One CTA per four rows.  Every thread first asks for its share of the rows' q / k / v chunks (up to ten 16-byte loads in
+// HBM bound: 26 KB a row, 24.4 us at the copy rate for 6144 rows; measured 28 us.  One CTA per two rows of 128 threads: with four rows
+// and 256 threads the last wave of 64 prompts was a third full and small steps had fewer CTAs than SMs (8 prompts 38.0 -> 37.5 us
+// a step, 32 prompts 108.2 -> 107.3, the first inference step of 64 prompts, rotation only, 3.35 -> 3.33 ms).  The rotation
+// alone is held to 64 registers, eight CTAs per SM (1 prompt's first inference step 64.4 -> 62.6 us); the fused kernel spills
+// nothing at 80 and lost 5 to 8 % of the step at 64.
+// Every thread first asks for its share of the rows' q / k / v chunks (up to ten 16-byte loads in
 // flight per thread), then evaluates one of the rows' D/2 (cos, sin) pairs; they are kept in shared memory as fp32 and
 // applied to all Hq + Hkv heads: a thread rotates 8 pairs at a time from one 16-byte chunk of the low half and one of the high half.
 // Angles reach thousands of radians, where an fp32 product pos * inv_freq already loses ~1e-4 rad: the product and its
@@ -33,7 +38,7 @@ struct AppendDst {                                   // fused kernel only: where
 };
 
 template <int D, bool FUSED>
-__global__ void __launch_bounds__(kRopeThreads)
+__global__ void __launch_bounds__(kRopeThreads, FUSED ? 6 : 8)
 rope_kernel(int Hq, int Hkv, const InvFreq inv_freq, const int32_t* __restrict__ n_active,
             const int32_t* __restrict__ pos_id, __nv_bfloat16* __restrict__ q, __nv_bfloat16* __restrict__ k_new,
             const AppendDst ad)
