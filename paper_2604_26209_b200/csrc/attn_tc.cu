@@ -324,6 +324,7 @@ hpd_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int G = p.G;
     if ((smem_u32(smem) & 1023u) != 0) {                 // swizzled tiles need 1024-byte alignment: refuse rather than misread
+        await_predecessors();
         if (threadIdx.x == 0 && p.a.dev_status) atomicOr(p.a.dev_status, HPD_S_BAD_TABLE);
         return;
     }
@@ -365,8 +366,13 @@ hpd_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         // microseconds or more, so one stage per iteration is ample for an L2 round trip.)
         reg_dealloc<kRegsIo>();
         const int x = warp == 0 ? 0 : 1;
-        const int n_units = p.hdr->n_work * p.a.g.Hkv;
         const int Hkv = p.a.g.Hkv;
+        // The pipeline's first unit is one of two, whichever way the units are laid over the SMs: both items are asked for together with
+        // the header that says how many there are (and which way it is), one round trip instead of two before the first copy.
+        const int first_spread = blockIdx.x + x * gridDim.x, first_pair = 2 * blockIdx.x + x;
+        const WorkItem it_spread = p.work[min(first_spread / Hkv, p.a.lay.work_cap - 1)];
+        const WorkItem it_pair = p.work[min(first_pair / Hkv, p.a.lay.work_cap - 1)];
+        const int n_units = p.hdr->n_work * Hkv;
         const int64_t cache_rows = static_cast<int64_t>(p.a.n_slots) * p.a.g.suffix_cap;
         uint32_t* ticket = const_cast<uint32_t*>(&p.hdr->ticket);
         UnitDesc& d = misc->desc[x];
@@ -402,7 +408,8 @@ hpd_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         };
         int w0 = fixed(0), w1 = fixed(1), w2 = fixed(2), w3 = fixed(3);
         auto item_of = [&](int w) { return p.work[min(w, max(n_units - 1, 0)) / Hkv]; };
-        WorkItem it2 = item_of(w2), it1 = item_of(w1), it0 = item_of(w0);
+        WorkItem it2 = item_of(w2), it1 = item_of(w1);
+        WorkItem it0 = (spread ? first_spread : first_pair) < n_units ? (spread ? it_spread : it_pair) : item_of(w0);
         int das1 = p.a.doc_active_start[it1.doc], dks1 = p.a.doc_kv_start[it1.doc];
         int das0 = p.a.doc_active_start[it0.doc], dks0 = p.a.doc_kv_start[it0.doc];
         // shared block of the unit's document: its id one stage ahead of its first row and length
@@ -780,7 +787,6 @@ hpd_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                         }
                     }
                 }
-                ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 // Probabilities go to tensor memory as bf16 pairs (column c holds keys 2c and 2c+1 of the row), over the
                 // first half of the row's own scores, from where the tensor core reads them as the A operand of O += P V.

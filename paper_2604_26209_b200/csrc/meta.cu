@@ -302,9 +302,8 @@ __device__ __forceinline__ void plan_block(int n_docs, int G, int Hkv, int n_sm,
     }
     __syncthreads();
     const bool enough = static_cast<long long>(s_whole) * Hkv >= n_sm;
-    // worth the sort only when the units differ: more than a quarter between the shortest and the longest (a split
-    // list always goes through the pass below: its chunks differ)
-    const bool differ = !enough || (s_cost_max > s_cost_min && (s_cost_max - s_cost_min) * 4 > s_cost_max);
+    // worth the sort only when the units differ: more than a quarter between the shortest and the longest, or the chunks of a split list
+    bool differ = s_cost_max > s_cost_min && (s_cost_max - s_cost_min) * 4 > s_cost_max;
     int cand = kCand - 1;                                // whole documents
     if (!enough) {
         if (warp < kCand) {                              // warp c weighs chunk size c
@@ -335,6 +334,7 @@ __device__ __forceinline__ void plan_block(int n_docs, int G, int Hkv, int n_sm,
         }
         __syncthreads();
         cand = s_choice;
+        differ |= s_prow[cand] > 0;
     }
 
     int parity = 0;
