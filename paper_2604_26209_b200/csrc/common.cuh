@@ -57,11 +57,10 @@ struct WsHeader {
     int32_t chunk_tokens;    // prefix tokens per work item (0: documents are not split)
     int32_t n_part_rows;     // partial rows in use
     int32_t any_split;       // 1 if some document is split (the merge kernel has work)
-    uint32_t ticket;         // dynamic scheduler: next work item
-    uint32_t finished;       // CTAs that have drained the list (the last one resets both)
+    uint32_t ticket;         // dynamic scheduler: next unit beyond the fixed rounds
     int32_t work_cap, part_cap;
     int32_t longest_first;   // 1 if the list is in descending order of the units' estimated duration
-    int32_t pad[23];
+    int32_t pad[24];
 };
 static_assert(sizeof(WsHeader) == 128, "header size");
 
