@@ -935,7 +935,7 @@ hpd_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
 // chain of L2 round trips, not of bytes).
 template <int D>
 __global__ void __launch_bounds__(256)
-hpd_merge_kernel(TcParams p, const DocSplit* __restrict__ split)
+hpd_merge_kernel(TcParams p, const DocSplit* split)
 {
     start_dependents();
     await_predecessors();

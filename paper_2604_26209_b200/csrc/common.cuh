@@ -158,6 +158,8 @@ int launch_attn_tc(const AttnArgs& a);       // tcgen05 / TMA kernel
 // await_predecessors() before its first access to global memory; that returns once the predecessor has completed and its
 // writes are visible.  Every kernel launched like this waits in all of its blocks, so "the predecessor has completed"
 // includes everything before it.
+// Such a kernel is resident while others still write what it will read: none of its pointer parameters is __restrict__, which would
+// promise that nothing else writes there during the kernel's life and so allow reads through the non-coherent path or above the wait.
 // ---------------------------------------------------------------------------------------------
 __device__ __forceinline__ void await_predecessors() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void start_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

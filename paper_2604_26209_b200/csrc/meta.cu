@@ -477,14 +477,14 @@ __device__ __forceinline__ uint32_t nonzero_bytes(uint32_t w) {
 
 __global__ void __launch_bounds__(kPlanThreads)
 meta_step_kernel(int n_docs, int n_slots, int32_t suffix_cap, int32_t pos_gap, int G, int Hkv, int n_sm,
-                 const int32_t* __restrict__ doc_prefix_len, const int32_t* __restrict__ doc_branch_cnt,
-                 const int32_t* __restrict__ slot_depth, const uint8_t* __restrict__ slot_alive,
-                 const int32_t* __restrict__ slot_vis /* nullable */,
-                 int32_t* __restrict__ doc_kv_start, int32_t* __restrict__ doc_slot_start, int32_t* __restrict__ doc_active_start,
-                 int32_t* __restrict__ active_slot, int32_t* __restrict__ doc_id, int32_t* __restrict__ branch_start,
-                 int32_t* __restrict__ pos_id, int32_t* __restrict__ suffix_off, int32_t* __restrict__ suffix_len,
-                 int32_t* __restrict__ prefix_vis /* nullable */,
-                 int32_t* __restrict__ n_active, WsHeader* __restrict__ hdr, WorkItem* __restrict__ work, DocSplit* __restrict__ split,
+                 const int32_t* doc_prefix_len, const int32_t* doc_branch_cnt,
+                 const int32_t* slot_depth, const uint8_t* slot_alive,
+                 const int32_t* slot_vis /* nullable */,
+                 int32_t* doc_kv_start, int32_t* doc_slot_start, int32_t* doc_active_start,
+                 int32_t* active_slot, int32_t* doc_id, int32_t* branch_start,
+                 int32_t* pos_id, int32_t* suffix_off, int32_t* suffix_len,
+                 int32_t* prefix_vis /* nullable */,
+                 int32_t* n_active, WsHeader* hdr, WorkItem* work, DocSplit* split,
                  int work_cap, int part_cap)
 {
     __shared__ int s_start[kStepDocs + 1];           // first slot of every document; block 0 turns it into its first row
@@ -615,12 +615,12 @@ constexpr int kPrefillThreads = 256;
 
 __global__ void __launch_bounds__(kPrefillThreads)
 prefill_meta_kernel(int n_docs, int G, int32_t pos_gap,
-                    const int32_t* __restrict__ doc_prefix_len, const int32_t* __restrict__ doc_branch_cnt,
-                    const int32_t* __restrict__ slot_vis,
-                    int32_t* __restrict__ doc_kv_start, int32_t* __restrict__ doc_slot_start,
-                    int32_t* __restrict__ tok_doc, int32_t* __restrict__ tok_pos, int32_t* __restrict__ tok_vis,
-                    int32_t* __restrict__ n_tokens, WsHeader* __restrict__ hdr, WorkItem* __restrict__ work,
-                    DocSplit* __restrict__ split, int work_cap, int part_cap)
+                    const int32_t* doc_prefix_len, const int32_t* doc_branch_cnt,
+                    const int32_t* slot_vis,
+                    int32_t* doc_kv_start, int32_t* doc_slot_start,
+                    int32_t* tok_doc, int32_t* tok_pos, int32_t* tok_vis,
+                    int32_t* n_tokens, WsHeader* hdr, WorkItem* work,
+                    DocSplit* split, int work_cap, int part_cap)
 {
     __shared__ int sm[kPrefillThreads / 32 + 1];
     __shared__ int s_kv[kPrefillDocs + 1], s_slot[kPrefillDocs + 1], s_item[kPrefillDocs + 1];

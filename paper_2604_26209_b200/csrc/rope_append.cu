@@ -39,8 +39,8 @@ struct AppendDst {                                   // fused kernel only: where
 
 template <int D, bool FUSED>
 __global__ void __launch_bounds__(kRopeThreads, FUSED ? 6 : 8)
-rope_kernel(int Hq, int Hkv, const InvFreq inv_freq, const int32_t* __restrict__ n_active,
-            const int32_t* __restrict__ pos_id, __nv_bfloat16* __restrict__ q, __nv_bfloat16* __restrict__ k_new,
+rope_kernel(int Hq, int Hkv, const InvFreq inv_freq, const int32_t* n_active,
+            const int32_t* pos_id, __nv_bfloat16* q, __nv_bfloat16* k_new,
             const AppendDst ad)
 {
     constexpr int HALF = D / 2;
@@ -232,9 +232,9 @@ const InvFreq& inv_freq_table(const hpd_geom& g)
 constexpr int kAdvanceThreads = 1024, kAdvanceRows = 8 * kAdvanceThreads;
 
 __global__ void __launch_bounds__(kAdvanceThreads)
-advance_kernel(int max_rows, int32_t suffix_cap, int32_t delimiter_id, const int32_t* __restrict__ n_active,
-               const int32_t* __restrict__ active_slot, const int32_t* __restrict__ token_id,
-               int32_t* __restrict__ slot_depth, uint8_t* __restrict__ slot_alive, int32_t* __restrict__ n_alive)
+advance_kernel(int max_rows, int32_t suffix_cap, int32_t delimiter_id, const int32_t* n_active,
+               const int32_t* active_slot, const int32_t* token_id,
+               int32_t* slot_depth, uint8_t* slot_alive, int32_t* n_alive)
 {
     start_dependents();
     await_predecessors();
@@ -244,10 +244,10 @@ advance_kernel(int max_rows, int32_t suffix_cap, int32_t delimiter_id, const int
         const int r = base + threadIdx.x;
         int stays = 0;
         if (r < n) {
-            const int s = active_slot[r];
+            const int s = active_slot[r], token = token_id[r];     // both loads before the stores
             const int d = min(slot_depth[s] + 1, suffix_cap);      // the step's token went into the slab (unless it was full)
             slot_depth[s] = d;
-            stays = token_id[r] != delimiter_id && d < suffix_cap;
+            stays = token != delimiter_id && d < suffix_cap;
             slot_alive[s] = static_cast<uint8_t>(stays);
         }
         live += __syncthreads_count(stays);
