@@ -20,6 +20,7 @@ void set_last_cuda_error(cudaError_t e);
     do {                                                     \
         cudaError_t e__ = (expr);                            \
         if (e__ != cudaSuccess) {                            \
+            (void)cudaGetLastError(); /* reported here, not by the next call as well */ \
             ::hpd::set_last_cuda_error(e__);                 \
             return HPD_E_CUDA;                               \
         }                                                    \
