@@ -54,11 +54,10 @@ template <typename T> bool convert(PyObject* o, T& out)
         out = static_cast<T>(t.data_ptr());
         return true;
     } else {
-        if (!PyLong_Check(o)) {
-            PyErr_SetString(PyExc_TypeError, "an integer is expected");
-            return false;
-        }
-        out = static_cast<T>(PyLong_AsUnsignedLongLongMask(o));      // as ctypes does
+        PyObject* n = PyNumber_Index(o);                             // integers and what stands for one (NumPy's, 0-d tensors); no floats
+        if (!n) return false;
+        out = static_cast<T>(PyLong_AsUnsignedLongLongMask(n));      // as ctypes does
+        Py_DECREF(n);
         return !PyErr_Occurred();
     }
 }

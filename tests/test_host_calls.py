@@ -1,4 +1,5 @@
 """Native marshalling of the per-step calls: what it refuses, before anything reaches the library (no GPU needed)."""
+import numpy as np
 import pytest
 import torch
 
@@ -23,3 +24,13 @@ def test_every_step_call_is_marshalled_natively():
 def test_refused_arguments(args, error):
     with pytest.raises(error):
         binding._calls().hpd_rope(*args)
+
+
+@pytest.mark.parametrize("n", [0, False, np.int32(0), np.int64(0), torch.tensor(0)])
+def test_sizes_may_be_any_integer(n):
+    """Whatever has an integer value passes, as it does through ctypes: the call gets as far as the current stream."""
+    if torch.cuda.is_available():
+        assert binding._calls().hpd_rope(GEOM, n, None, None, None, None) == 0
+    else:
+        with pytest.raises(RuntimeError):
+            binding._calls().hpd_rope(GEOM, n, None, None, None, None)
