@@ -504,7 +504,9 @@ meta_step_kernel(int n_docs, int n_slots, int32_t suffix_cap, int32_t pos_gap, i
     // ---- everything that is read from memory is asked for here ----
     const int depth = mine ? slot_depth[s] : 0;
     const int my_vis = (slot_vis && mine) ? slot_vis[s] : 0;
-    int l = t < n_docs ? doc_prefix_len[t] : 0, c = t < n_docs ? doc_branch_cnt[t] : 0;
+    // a count outside [0, n_slots] cannot be right and is clamped: the first slots below index shared memory
+    auto count_of = [&](int d) { return min(max(doc_branch_cnt[d], 0), n_slots); };
+    int l = t < n_docs ? doc_prefix_len[t] : 0, c = t < n_docs ? count_of(t) : 0;
     uint32_t m[2] = {0u, 0u};                        // live flags of slots [64 t, 64 t + 64)
     if ((reinterpret_cast<uintptr_t>(slot_alive) & 15) == 0 && (t + 1) * 64 <= n_slots) {
         const uint4* v = reinterpret_cast<const uint4*>(slot_alive) + t * 4;
@@ -529,7 +531,7 @@ meta_step_kernel(int n_docs, int n_slots, int32_t suffix_cap, int32_t pos_gap, i
         if (base > 0) {
             const int d = base + t;
             l = d < n_docs ? doc_prefix_len[d] : 0;
-            c = d < n_docs ? doc_branch_cnt[d] : 0;
+            c = d < n_docs ? count_of(d) : 0;
         }
         if (base == 0 && lane == 31) s_cnt[warp] = pop_incl;
         long long tot;

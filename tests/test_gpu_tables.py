@@ -37,3 +37,22 @@ def test_tables_at_block_edges(docs, slots, misaligned):
     for name in capi.Meta.TABLES:
         w = getattr(want, name)
         assert np.array_equal(getattr(m, name).cpu().numpy()[:len(w)], w), name
+
+
+@pytest.mark.parametrize("docs", [3, 1500])
+@pytest.mark.parametrize("wrong", [-1, -40, -2**31, 2**31 - 1])
+def test_counts_outside_the_slots_stay_inside_the_tables(docs, wrong):
+    """A count no document can have is taken as 0 or as all slots: first slots ascend, every row range lies inside the rows."""
+    from paper_2604_26209_b200 import binding as B
+    slots = 2 * docs
+    cnt = np.full(docs, 2, np.int32)
+    cnt[docs // 2] = wrong
+    g = synth.Geom(Hq=2, Hkv=1, D=64, rope_theta=10000.0, sm_scale=0.125, suffix_cap=4)
+    m = B.MetaTables.alloc(g, docs, slots, docs)
+    dev = lambda a: torch.from_numpy(a).cuda()                        # noqa: E731
+    B.hpd_build_meta(g, docs, slots, dev(np.ones(docs, np.int32)), dev(cnt), dev(np.zeros(slots, np.int32)), dev(np.ones(slots, np.uint8)), 0, m)
+    torch.cuda.synchronize()
+    first = np.concatenate([[0], np.cumsum(np.clip(cnt, 0, slots))])
+    assert int(m.n_active.item()) == slots
+    assert np.array_equal(m.doc_slot_start.cpu().numpy()[:docs + 1], first)
+    assert np.array_equal(m.doc_active_start.cpu().numpy()[:docs + 1], np.concatenate([np.minimum(first[:-1], slots), [slots]]))
