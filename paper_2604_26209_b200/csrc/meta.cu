@@ -475,6 +475,9 @@ __device__ __forceinline__ uint32_t nonzero_bytes(uint32_t w) {
     return ((__vcmpne4(w, 0u) & 0x08040201u) * 0x01010101u) >> 24;
 }
 
+// SHIFTED: the live flags do not begin on a 16-byte address (a slice of a larger buffer).  A kernel of its own, because the
+// other form lost 1 to 7 % with both in one; single bytes took 29 us at 65536 slots, the pieces take 14.
+template <bool SHIFTED>
 __global__ void __launch_bounds__(kPlanThreads)
 meta_step_kernel(int n_docs, int n_slots, int32_t suffix_cap, int32_t pos_gap, int G, int Hkv, int n_sm,
                  const int32_t* doc_prefix_len, const int32_t* doc_branch_cnt,
@@ -508,7 +511,39 @@ meta_step_kernel(int n_docs, int n_slots, int32_t suffix_cap, int32_t pos_gap, i
     auto count_of = [&](int d) { return min(max(doc_branch_cnt[d], 0), n_slots); };
     int l = t < n_docs ? doc_prefix_len[t] : 0, c = t < n_docs ? count_of(t) : 0;
     uint32_t m[2] = {0u, 0u};                        // live flags of slots [64 t, 64 t + 64)
-    if ((reinterpret_cast<uintptr_t>(slot_alive) & 15) == 0 && (t + 1) * 64 <= n_slots) {
+    if constexpr (SHIFTED) {
+        // five pieces of 16 slots, the first from sh slots earlier, one load each where they lie inside the flags and single bytes at the two ends
+        const int sh = static_cast<int>(reinterpret_cast<uintptr_t>(slot_alive) & 15), q0 = t * 64 - sh;
+        if (q0 < n_slots) {
+            uint4 w[5];
+            unsigned long long lo = 0;                   // slots q0 .. q0 + 63
+            uint32_t hi = 0, ends = 0;                   // slots from q0 + 64; pieces that lie inside in part
+#pragma unroll
+            for (int i = 0; i < 5; ++i) {
+                const int q = q0 + 16 * i;
+                w[i] = make_uint4(0, 0, 0, 0);
+                if (q >= 0 && q + 16 <= n_slots) w[i] = *reinterpret_cast<const uint4*>(slot_alive + q);
+                else if (q < n_slots) ends |= 1u << i;
+            }
+#pragma unroll 1
+            while (ends) {
+                const int i = __ffs(ends) - 1, q = q0 + 16 * i;
+                ends &= ends - 1;
+                uint32_t f = 0;
+#pragma unroll
+                for (int b = 0; b < 16; ++b)
+                    if (q + b >= 0 && q + b < n_slots && slot_alive[q + b]) f |= 1u << b;
+                if (i < 4) lo |= static_cast<unsigned long long>(f) << (16 * i); else hi |= f;
+            }
+#pragma unroll
+            for (int i = 0; i < 5; ++i) {
+                const uint32_t f = nonzero_bytes(w[i].x) | nonzero_bytes(w[i].y) << 4 | nonzero_bytes(w[i].z) << 8 | nonzero_bytes(w[i].w) << 12;
+                if (i < 4) lo |= static_cast<unsigned long long>(f) << (16 * i); else hi |= f;
+            }
+            lo = lo >> sh | static_cast<unsigned long long>(hi) << (64 - sh);
+            m[0] = static_cast<uint32_t>(lo); m[1] = static_cast<uint32_t>(lo >> 32);
+        }
+    } else if ((t + 1) * 64 <= n_slots) {
         const uint4* v = reinterpret_cast<const uint4*>(slot_alive) + t * 4;
         uint4 w[4];
 #pragma unroll
@@ -746,7 +781,7 @@ int launch_build_meta(const hpd_geom& g, int n_docs, int n_slots, const int32_t*
     // one launch up to 4096 documents and 65536 slots: what a block can hold in shared memory (45 KB) and count in 16 bits
     if (n_docs <= kStepDocs && n_slots <= kStepSlots) {
         const int blocks = 1 + (n_slots + kPlanThreads - 1) / kPlanThreads;
-        HPD_CUDA_TRY(launch_chained(meta_step_kernel, blocks, kPlanThreads, 0, stream,
+        HPD_CUDA_TRY(launch_chained(aligned16(slot_alive) ? meta_step_kernel<false> : meta_step_kernel<true>, blocks, kPlanThreads, 0, stream,
             n_docs, n_slots, g.suffix_cap, pos_gap, g.Hq / g.Hkv, g.Hkv, n_sm, doc_prefix_len, doc_branch_cnt, slot_depth,
             slot_alive, slot_vis, doc_kv_start, doc_slot_start, doc_active_start, active_slot, doc_id, branch_start, pos_id,
             suffix_off, suffix_len, prefix_vis, n_active, hdr, work, split, lay.work_cap, lay.part_cap));

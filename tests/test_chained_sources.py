@@ -10,7 +10,7 @@ def _chained():
     """(name, parameter list) of every kernel handed to launch_chained."""
     text = "\n".join(open(f).read() for f in sorted(glob.glob(os.path.join(CSRC, "*.cu"))))
     found = []
-    for name in sorted(set(re.findall(r"launch_chained\((\w+)", text))):
+    for name in sorted(set(re.findall(r"launch_chained\((?:[^,]*\? *)?(\w+)", text))):
         m = re.search(r"__global__[^;{]*?\b" + name + r"\((.*?)\)\s*\{.*?await_predecessors\(\);", text, re.S)
         assert m, f"{name}: no definition with a wait"
         found.append((name, m.group(1)))

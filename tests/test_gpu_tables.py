@@ -56,3 +56,9 @@ def test_counts_outside_the_slots_stay_inside_the_tables(docs, wrong):
     assert int(m.n_active.item()) == slots
     assert np.array_equal(m.doc_slot_start.cpu().numpy()[:docs + 1], first)
     assert np.array_equal(m.doc_active_start.cpu().numpy()[:docs + 1], np.concatenate([np.minimum(first[:-1], slots), [slots]]))
+
+
+@pytest.mark.parametrize("offset", [2, 7, 8, 15])
+@pytest.mark.parametrize("docs,slots", [(1, 1), (2, 17), (3, 33), (5, 64), (40, 1023), (9, 65536)])
+def test_live_flags_at_any_address(docs, slots, offset):
+    test_tables_at_block_edges(docs, slots, offset)
