@@ -7,19 +7,18 @@ CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
 
 
 def _chained():
-    """(name, parameter list) of every kernel handed to launch_chained."""
+    """{name: parameter list} of every kernel that waits for its predecessors itself."""
     text = "\n".join(open(f).read() for f in sorted(glob.glob(os.path.join(CSRC, "*.cu"))))
-    found = []
-    for name in sorted(set(re.findall(r"launch_chained\((?:[^,]*\? *)?(\w+)", text))):
-        m = re.search(r"__global__[^;{]*?\b" + name + r"\((.*?)\)\s*\{.*?await_predecessors\(\);", text, re.S)
-        assert m, f"{name}: no definition with a wait"
-        found.append((name, m.group(1)))
+    found = {}
+    for kernel in re.split(r"(?=__global__)", text)[1:]:
+        name, params = re.match(r"__global__[^;{]*?\b(\w+_kernel)\((.*?)\)\s*\{", kernel, re.S).groups()
+        if "await_predecessors();" in kernel:
+            found[name] = params
     return found
 
 
 def test_chained_kernels_have_no_restrict_parameters():
     kernels = _chained()
-    assert [k[0] for k in kernels] == ["advance_kernel", "hpd_attn_tc_kernel", "hpd_merge_kernel", "meta_step_kernel", "prefill_meta_kernel",
-                                       "rope_kernel"]
-    for name, params in kernels:
+    assert set(kernels) == {"advance_kernel", "hpd_attn_tc_kernel", "hpd_merge_kernel", "meta_step_kernel", "prefill_meta_kernel", "rope_kernel"}
+    for name, params in kernels.items():
         assert "__restrict__" not in params, f"{name}: a predecessor may still write what a __restrict__ parameter points to"

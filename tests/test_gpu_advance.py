@@ -28,3 +28,9 @@ def test_advance_at_block_edges(rows, idle):
     torch.cuda.synchronize()
     assert int(count.item()) == int(a[slot[:rows]].sum())
     assert np.array_equal(gd.cpu().numpy()[:n], d) and np.array_equal(ga.cpu().numpy()[:n], a)
+
+
+@pytest.mark.parametrize("rows", [2047, 2048, 2049, 4095, 4096, 4097, 6145])
+def test_advance_at_pass_edges(rows):
+    test_advance_at_block_edges(rows, 0)
+    test_advance_at_block_edges(rows, 5000)          # idle entries past the one-block limit
