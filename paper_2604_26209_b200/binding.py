@@ -2,7 +2,7 @@
 
 Argument marshalling only: tensors are passed as raw device pointers together with the current
 CUDA stream; every step of the path runs in the library's kernels.  PyTorch is used for device
-memory and streams.  The calls of a step go through ``_host.so`` (native marshalling, ``csrc/host.cpp``: ctypes took longer
+memory and streams.  The calls of a step go through ``_host`` (native marshalling, ``csrc/host.cpp``: ctypes took longer
 than the GPU for a small step), the others through ctypes.  Both libraries must be present -- there is no fallback;
 ``load()`` raises if they have not been built (``python -m paper_2604_26209_b200.build``).
 """
@@ -14,6 +14,8 @@ from dataclasses import dataclass
 from typing import Optional
 
 import torch
+
+from . import build
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(HERE, "libhpd.so")
@@ -89,11 +91,16 @@ def load() -> C.CDLL:
         lib.std_attn_decode_static_max_bytes.argtypes = []
         lib.std_attn_decode_static.restype = C.c_int
         lib.std_attn_decode_static.argtypes = [C.POINTER(HpdGeom), C.c_int, C.c_int, C.c_longlong] + [vp] * 8 + [vp]
+        key = build.host_key()
         try:
             from . import _host as host
         except ImportError as e:
-            raise HpdError(f"_host.so is missing or does not fit this interpreter: build it with `python -m "
+            raise HpdError(f"the native calls (_host) are missing or do not load: build them with `python -m "
                            f"paper_2604_26209_b200.build` ({e})") from e
+        built_for = getattr(host, "BUILT_FOR", "an unknown torch")
+        if built_for != key:
+            raise HpdError(f"the native calls (_host) were built for {built_for}, this is {key}: build them with `python -m "
+                           "paper_2604_26209_b200.build`")
         for name in host.ENTRIES:
             host.set_address(name, C.cast(getattr(lib, name), C.c_void_p).value)
         _host = host

@@ -1,4 +1,4 @@
-"""Compile the CUDA sources in-tree into ``libhpd.so`` for sm_100a and the Python side of its calls into ``_host.so``
+"""Compile the CUDA sources in-tree into ``libhpd.so`` for sm_100a and the Python side of its calls into ``_host`` (for this interpreter)
 (``python -m paper_2604_26209_b200.build``)."""
 from __future__ import annotations
 
@@ -13,7 +13,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libhpd.so")
-HOST = os.path.join(HERE, "_host.so")
+HOST = os.path.join(HERE, "_host" + sysconfig.get_config_var("EXT_SUFFIX"))
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std=c++17",
               "-Xcompiler", "-fPIC", "-Xcompiler", "-Wall", "-Xptxas", "-v"]
@@ -46,10 +46,17 @@ def _compile(src: str, verbose: bool) -> str:
     return obj
 
 
+def host_key() -> str:
+    """What the native calls are compiled against: they use the interpreter's C API and torch's C++ classes."""
+    import torch
+    return f"torch {torch.__version__} {torch.version.git_version} abi{int(torch._C._GLIBCXX_USE_CXX11_ABI)}, {sysconfig.get_config_var('EXT_SUFFIX')}"
+
+
 def _build_host() -> None:
-    src = os.path.join(CSRC, "host.cpp")
+    src, key_file, key = os.path.join(CSRC, "host.cpp"), os.path.join(OBJ, "_host.key"), host_key()
     if os.path.exists(HOST) and os.path.getmtime(HOST) >= max(os.path.getmtime(src), _deps_mtime()):
-        return
+        if os.path.exists(key_file) and open(key_file).read() == key:
+            return
     import torch
     root = os.path.dirname(torch.__file__)
     cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
@@ -57,6 +64,7 @@ def _build_host() -> None:
            os.path.join(cuda, "include"), sysconfig.get_paths()["include"]]
     tmp = HOST + f".tmp{os.getpid()}"
     cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-Wall", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           f'-DHPD_BUILT_FOR="{key}"',
            *["-isystem" + i for i in inc], src, "-o", tmp, "-L" + os.path.join(root, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu",
            "-ltorch_python"]
     res = subprocess.run(cmd, capture_output=True, text=True)
@@ -64,6 +72,8 @@ def _build_host() -> None:
         sys.stderr.write(res.stdout + res.stderr)
         raise RuntimeError(f"g++ failed on {src}")
     os.replace(tmp, HOST)
+    with open(key_file, "w") as f:
+        f.write(key)
 
 
 def build(force: bool = False, verbose: bool = False) -> str:

@@ -138,5 +138,6 @@ PyMODINIT_FUNC PyInit__host(void)
     HPD_ENTRIES(X)
 #undef X
     if (!names || PyModule_AddObject(m, "ENTRIES", names) < 0) return nullptr;
+    if (PyModule_AddStringConstant(m, "BUILT_FOR", HPD_BUILT_FOR) < 0) return nullptr;
     return m;
 }
