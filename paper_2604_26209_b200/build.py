@@ -55,8 +55,10 @@ def host_key() -> str:
 def _build_host() -> None:
     src, key_file, key = os.path.join(CSRC, "host.cpp"), os.path.join(OBJ, "_host.key"), host_key()
     if os.path.exists(HOST) and os.path.getmtime(HOST) >= max(os.path.getmtime(src), _deps_mtime()):
-        if os.path.exists(key_file) and open(key_file).read() == key:
-            return
+        if os.path.exists(key_file):
+            with open(key_file) as f:
+                if f.read() == key:
+                    return
     import torch
     root = os.path.dirname(torch.__file__)
     cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
