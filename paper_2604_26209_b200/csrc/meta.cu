@@ -507,9 +507,7 @@ meta_step_kernel(int n_docs, int n_slots, int32_t suffix_cap, int32_t pos_gap, i
     // ---- everything that is read from memory is asked for here ----
     const int depth = mine ? slot_depth[s] : 0;
     const int my_vis = (slot_vis && mine) ? slot_vis[s] : 0;
-    // a count outside [0, n_slots] cannot be right and is clamped: the first slots below index shared memory
-    auto count_of = [&](int d) { return min(max(doc_branch_cnt[d], 0), n_slots); };
-    int l = t < n_docs ? doc_prefix_len[t] : 0, c = t < n_docs ? count_of(t) : 0;
+    int l = t < n_docs ? doc_prefix_len[t] : 0, c = t < n_docs ? doc_branch_cnt[t] : 0;
     uint32_t m[2] = {0u, 0u};                        // live flags of slots [64 t, 64 t + 64)
     if constexpr (SHIFTED) {
         // five pieces of 16 slots, the first from sh slots earlier, one load each where they lie inside the flags and single bytes at the two ends
@@ -566,11 +564,12 @@ meta_step_kernel(int n_docs, int n_slots, int32_t suffix_cap, int32_t pos_gap, i
         if (base > 0) {
             const int d = base + t;
             l = d < n_docs ? doc_prefix_len[d] : 0;
-            c = d < n_docs ? count_of(d) : 0;
+            c = d < n_docs ? doc_branch_cnt[d] : 0;
         }
         if (base == 0 && lane == 31) s_cnt[warp] = pop_incl;
         long long tot;
-        const long long ex = scan_words(words(l, c), s_scan[(base / kPlanThreads) & 1], tot);
+        // a count outside [0, n_slots] cannot be right and is clamped: the first slots index shared memory below
+        const long long ex = scan_words(words(l, min(max(c, 0), n_slots)), s_scan[(base / kPlanThreads) & 1], tot);
         const int d = base + t;
         if (d < n_docs) {
             const int kv0 = run_kv + word_lo(ex), sl0 = run_sl + word_hi(ex);
