@@ -12,8 +12,8 @@ namespace hpd {
 namespace {
 
 constexpr int kRopeThreads = 128;
-constexpr unsigned kOneWave = 6 * 148;               // CTAs of the fused kernel that are resident at once (80 registers x 128 threads)
 constexpr int kRopeRows = 2;                         // rows per CTA: 2 x 64 angles give every thread one to evaluate
+template <bool FUSED> constexpr int kRopeResident = FUSED ? 6 : 8;   // CTAs of an SM (registers: 80 / 64 x 128 threads)
 
 // HBM bound: 26 KB a row, 24.4 us at the copy rate for 6144 rows; measured 28 us.  One CTA per two rows of 128 threads: with four rows
 // and 256 threads the last wave of 64 prompts was a third full and small steps had fewer CTAs than SMs (8 prompts 38.0 -> 37.5 us
@@ -38,10 +38,10 @@ struct AppendDst {                                   // fused kernel only: where
 };
 
 template <int D, bool FUSED>
-__global__ void __launch_bounds__(kRopeThreads, FUSED ? 6 : 8)
+__global__ void __launch_bounds__(kRopeThreads, kRopeResident<FUSED>)
 rope_kernel(int Hq, int Hkv, const InvFreq inv_freq, const int32_t* n_active,
             const int32_t* pos_id, __nv_bfloat16* q, __nv_bfloat16* k_new,
-            const AppendDst ad)
+            const AppendDst ad, unsigned one_wave /* CTAs that are resident at once */)
 {
     constexpr int HALF = D / 2;
     constexpr int CHUNKS = HALF / 8;                 // 16-byte chunks per half
@@ -52,8 +52,9 @@ rope_kernel(int Hq, int Hkv, const InvFreq inv_freq, const int32_t* n_active,
     __shared__ long long s_dst[R];
     const int r0 = blockIdx.x * R;
     // the attention's CTAs take an SM each: they may come early only where they cannot keep rows of this kernel waiting (decode
-    // loop of 16 prompts 5.58 -> 5.52 ms; at 64 prompts, 1536 CTAs, it costs 5 us of 186)
-    if (gridDim.x <= kOneWave) start_dependents();
+    // loop of 16 prompts 5.58 -> 5.52 ms; at 64 prompts, 1536 CTAs, it costs 5 us of 186; first inference step of 1750 to 2300
+    // tokens, a wave of the unfused kernel but more than one of the fused, 46.5 -> 45.5 and 63.3 -> 62.3 us)
+    if (gridDim.x <= one_wave) start_dependents();
     await_predecessors();
     const int na = *n_active;
     if (r0 >= na) return;
@@ -305,6 +306,17 @@ merge_lse_kernel(int Hq, int max_rows, const int32_t* __restrict__ n_active,
     if (lse && lane == 0) lse[w] = out_l;
 }
 
+template <bool FUSED>
+int launch_rotation(const hpd_geom& g, int max_rows, const int32_t* n_active, const int32_t* pos_id, __nv_bfloat16* q,
+                    __nv_bfloat16* k_new, const AppendDst& ad, cudaStream_t stream)
+{
+    const unsigned blocks = (static_cast<unsigned>(max_rows) + kRopeRows - 1) / kRopeRows;
+    const unsigned one_wave = static_cast<unsigned>(kRopeResident<FUSED> * sm_count());
+    HPD_CUDA_TRY(launch_chained(g.D == 128 ? rope_kernel<128, FUSED> : rope_kernel<64, FUSED>, blocks, kRopeThreads, 0, stream,
+                                g.Hq, g.Hkv, inv_freq_table(g), n_active, pos_id, q, k_new, ad, one_wave));
+    return HPD_OK;
+}
+
 }  // namespace
 
 int launch_merge_lse(const hpd_geom& g, int max_rows, const int32_t* n_active, const __nv_bfloat16* o_a, const float* lse_a,
@@ -338,14 +350,7 @@ int launch_rope(const hpd_geom& g, int max_rows, const int32_t* n_active, const 
                 __nv_bfloat16* q, __nv_bfloat16* k_new, cudaStream_t stream)
 {
     if (max_rows <= 0) return HPD_OK;
-    const InvFreq& c = inv_freq_table(g);
-    const AppendDst none{};
-    if (g.D == 128)
-        HPD_CUDA_TRY(launch_chained(rope_kernel<128, false>, (max_rows + kRopeRows - 1) / kRopeRows, kRopeThreads, 0, stream, g.Hq, g.Hkv, c, n_active, pos_id, q, k_new, none));
-    else
-        HPD_CUDA_TRY(launch_chained(rope_kernel<64, false>, (max_rows + kRopeRows - 1) / kRopeRows, kRopeThreads, 0, stream, g.Hq, g.Hkv, c, n_active, pos_id, q, k_new, none));
-    HPD_CUDA_TRY(cudaGetLastError());
-    return HPD_OK;
+    return launch_rotation<false>(g, max_rows, n_active, pos_id, q, k_new, AppendDst{}, stream);
 }
 
 int launch_rope_append(const hpd_geom& g, int max_rows, int n_slots, const int32_t* n_active, const int32_t* pos_id,
@@ -354,15 +359,9 @@ int launch_rope_append(const hpd_geom& g, int max_rows, int n_slots, const int32
                        cudaStream_t stream)
 {
     if (max_rows <= 0) return HPD_OK;
-    const InvFreq& c = inv_freq_table(g);
     const AppendDst ad{g.suffix_cap, static_cast<int64_t>(n_slots) * g.suffix_cap, suffix_off, suffix_len, v_new,
                        suffix_k, suffix_v, dev_status};
-    if (g.D == 128)
-        HPD_CUDA_TRY(launch_chained(rope_kernel<128, true>, (max_rows + kRopeRows - 1) / kRopeRows, kRopeThreads, 0, stream, g.Hq, g.Hkv, c, n_active, pos_id, q, k_new, ad));
-    else
-        HPD_CUDA_TRY(launch_chained(rope_kernel<64, true>, (max_rows + kRopeRows - 1) / kRopeRows, kRopeThreads, 0, stream, g.Hq, g.Hkv, c, n_active, pos_id, q, k_new, ad));
-    HPD_CUDA_TRY(cudaGetLastError());
-    return HPD_OK;
+    return launch_rotation<true>(g, max_rows, n_active, pos_id, q, k_new, ad, stream);
 }
 
 int launch_kv_append(const hpd_geom& g, int max_rows, int n_slots, const int32_t* n_active, const int32_t* suffix_off,
