@@ -15,6 +15,13 @@
  *     with the shapes stated.
  *   - every call only ENQUEUES work on `stream` (a cudaStream_t passed as void*) and never
  *     synchronises.  Sizes that change per step (n_active) are read on the device.
+ *   - kernels are launched chained (programmatic stream serialisation): one may be resident before its
+ *     predecessor in the stream has ended, and waits for it before it touches device memory.  Ordinary
+ *     launches, copies and events around the calls are ordered as always.  A caller's own kernel that is launched
+ *     programmatically BEHIND a call may start before that call has ended: it has to wait
+ *     (cudaGridDependencySynchronize) before it touches anything that this or an earlier call in the
+ *     stream reads or writes.  One IN FRONT of a call has to wait in all of its blocks, too: a call
+ *     waits for its predecessor only, and takes that to include everything before it.
  *   - problems detected on the device set bits (HPD_S_*) in the caller's `dev_status` word
  *     with the offending access suppressed; kernels never trap.
  *   - documents are numbered globally in prompt order; "slots" are all branches ever admitted,
