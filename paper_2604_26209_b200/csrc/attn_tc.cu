@@ -154,9 +154,8 @@ __device__ __forceinline__ bool mbar_wait_warp(unsigned long long* bar, uint32_t
     return __all_sync(0xffffffffu, mbar_wait(bar, parity, misc));
 }
 
-// One lane of the converged warp.  The compiler knows that what it guards runs in a single thread and keeps the operands of
-// the tensor-core instructions in uniform registers; behind lane == 0 it moves them there one by one for every instruction (issuing
-// eight of them took ~1200 cycles instead of ~300; attention of 64 prompts 156 -> 153 us, first inference step 3.48 -> 3.33 ms).
+// One lane of the converged warp.  Measured against lane == 0: issuing eight tensor-core instructions ~300 cycles instead of ~1200,
+// attention of 64 prompts 156 -> 153 us, first inference step 3.48 -> 3.33 ms.
 __device__ __forceinline__ bool elect_one() {
     uint32_t p;
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
