@@ -149,3 +149,83 @@ def test_calls_behind_events_copies_and_ordinary_kernels(direct):
         mx, mean = err_stats(out["o"][:n].float().numpy(), want.o)
         assert mx <= 2e-2 and mean <= 2e-3, (mx, mean)
         assert np.max(np.abs(out["lse"][:n].numpy() - want.lse)) <= 2e-2
+
+
+@pytest.mark.parametrize("side", ["copy", "kernel"])
+def test_captured_calls_behind_a_join_of_two_streams(side):
+    """A graph in which each call also depends on another stream's copy or kernel that writes its inputs, against the step without them."""
+    from paper_2604_26209_b200 import runtime
+    s = synth.config_custom("join", Hq=8, Hkv=2, D=128, theta=10000.0, cap=6, prefix_lens=[300] * 16, branch_cnts=[8] * 16, depth_hi=5, seed=21,
+                            alive_frac=0.7)
+    tb = synth.make_tensors(s)
+    meta, want = oracle_step(s, tb)
+    act = np.concatenate([meta.active_slot[:meta.n_active], np.setdiff1d(np.arange(s.n_slots), meta.active_slot[:meta.n_active])])
+    db = runtime.DeviceBatch(s, tb)
+    inputs = [(db.q, tb["q"][act]), (db.k_new, tb["k_new"][act]), (db.v_new, tb["v_new"][act])]
+    inputs = [(t, torch.from_numpy(np.ascontiguousarray(a).view(np.int16)).cuda().view(torch.bfloat16).reshape(t.shape)) for t, a in inputs]
+    tables = [(db.slot_depth, db.slot_depth.clone()), (db.slot_alive, db.slot_alive.clone())]
+    write = (lambda t, a: t.copy_(a)) if side == "copy" else (lambda t, a: torch.mul(a, 1, out=t))    # a memcpy node, a kernel node
+    db.step()
+    other = torch.cuda.Stream()
+    graph = torch.cuda.CUDAGraph()
+
+    def beside(pairs):
+        main = torch.cuda.current_stream()
+        other.wait_stream(main)
+        with torch.cuda.stream(other):
+            for t, a in pairs:
+                write(t, a)
+        return lambda: main.wait_stream(other)
+
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        beside(tables)()
+        join = beside(inputs)
+        db.build_meta()
+        join()
+        db.rope_append()
+        join = beside([(db.lse, torch.zeros_like(db.lse))])
+        join()
+        db.attn(True)
+    for _ in range(3):
+        db.q.zero_(); db.k_new.zero_(); db.v_new.zero_(); db.o.zero_(); db.slot_alive.zero_(); db.slot_depth.fill_(1)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert db.status() == 0 and int(db.meta.n_active.item()) == meta.n_active
+        mx, mean = err_stats(synth.bf16_bits_to_f32(runtime.bits_of(db.o))[:meta.n_active], want.o)
+        assert mx <= 2e-2 and mean <= 2e-3, (mx, mean)
+        assert np.max(np.abs(db.lse.cpu().numpy()[:meta.n_active] - want.lse)) <= 2e-2
+
+
+@pytest.mark.parametrize("tokens", [40, 900, 5000])      # a few CTAs, about one wave of the rotation, more than one
+def test_back_to_back_first_steps_equal_synchronised_ones(tokens):
+    """Two first inference steps of two layers, with nothing between the calls, bit for bit as with a wait after each."""
+    from paper_2604_26209_b200 import binding as B
+    g = synth.Geom(Hq=8, Hkv=2, D=128, rope_theta=10000.0, sm_scale=128 ** -0.5, suffix_cap=8)
+    L = torch.tensor([tokens // 3, tokens - tokens // 3], dtype=torch.int32, device="cuda")
+    vis = torch.tensor([tokens // 6, tokens // 3, tokens // 5, tokens // 2], dtype=torch.int32, device="cuda")
+    cnt = torch.tensor([2, 2], dtype=torch.int32, device="cuda")
+    gen = torch.Generator(device="cuda").manual_seed(tokens)
+    start = [torch.randn(tokens, h, 128, device="cuda", generator=gen).to(torch.bfloat16) for _ in range(2 * LAYERS) for h in (8, 2, 2)]
+    t = B.PrefillTables.alloc(g, 2, tokens)
+
+    def run(wait):
+        for x in (t.doc_kv_start, t.doc_slot_start, t.tok_doc, t.tok_pos, t.tok_vis, t.n_tokens, t.workspace):
+            x.zero_()
+        work = [x.clone() for x in start]
+        outs = [torch.zeros_like(start[0]) for _ in range(2 * LAYERS)]
+        sync = torch.cuda.synchronize if wait else (lambda: None)
+        torch.cuda.synchronize()
+        for step in range(2):
+            B.hpd_prefill_meta(g, 2, 4, tokens, L, cnt, vis, 8, t); sync()
+            for l in range(step * LAYERS, (step + 1) * LAYERS):
+                q, k, v = work[3 * l:3 * l + 3]
+                B.hpd_rope(g, tokens, t.n_tokens, t.tok_pos, q, k); sync()
+                B.hpd_prefill_attn(g, 2, tokens, q, k, v, L, t, outs[l]); sync()
+        torch.cuda.synchronize()
+        assert int(t.dev_status.item()) == 0
+        return [x.view(torch.int16) for x in work + outs] + [x.clone() for x in (t.tok_doc, t.tok_pos, t.tok_vis, t.n_tokens)]
+
+    want = run(True)
+    for _ in range(3):
+        assert all(torch.equal(a, b) for a, b in zip(run(False), want))
