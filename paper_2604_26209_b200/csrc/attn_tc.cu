@@ -17,7 +17,8 @@
 // tiles and an output accumulator (tensor memory), and these warps:
 //
 //   warp 0 / 3    scheduler and TMA producer: draws the pipeline's units, publishes their
-//                 descriptors, issues Q, K and V tiles (prefix: lane 0; suffix boxes: all lanes)
+//                 descriptors, issues Q, K and V tiles (prefix: lane 0; suffix boxes: all lanes);
+//                 in the position-order decode warps 12 / 14 issue the K tiles and 13 / 15 the V tiles
 //   warp 1 / 2    MMA issuer: S = Q K^T (both operands in shared memory), two tiles ahead of the
 //                 softmax, and O += P V (P in tensor memory, V in shared memory); tcgen05.mma
 //   warps 4-7 /   softmax: one thread per row: S from TMEM, online max/sum, P as bf16 pairs written
@@ -39,8 +40,12 @@ namespace hpd {
 
 namespace {
 
-constexpr int kWarps = 12;
-constexpr int kThreads = kWarps * 32;
+// What a launch attends (template parameter): own document and branch; the same with a block shared by several documents in front;
+// position-order mask over a group's prefix and branch caches; position-order mask over prompts alone (first inference step).
+enum Mode { kOwn, kBlock, kOrder, kPrefill };
+// The position-order decode has four more warps, which copy K and V tiles (the reason stands at the kernel).
+template <int MODE> constexpr bool kCopyWarps = MODE == kOrder;
+template <int MODE> constexpr int kThreadsOf = kCopyWarps<MODE> ? 512 : 384;
 constexpr int kM = 128;                    // rows of a tile
 constexpr int kN = 64;                     // keys of a tile
 constexpr int kQHalf = kM * 128;           // one 64-element half of the Q tile: 128 rows x 128 B
@@ -52,13 +57,14 @@ constexpr long long kWaitCycles = 4000000000ll;   // ~2 s at 2 GHz
 // TMEM columns of one pipeline (the second pipeline's start 256 columns further): two score tiles of 64 columns (the
 // probabilities of a tile, bf16 pairs, overwrite the first 32 columns of its scores) and the output accumulator
 constexpr uint32_t kColPipe = 256, kColS = 0, kColO = 128;
-// registers per thread after the warpgroups have traded them (3 x 128 threads, 168 each at launch)
-constexpr int kRegsIo = 104, kRegsSoftmax = 200;
-// setmaxnreg only moves registers inside the CTA's own allocation (168 x 384 threads at launch): a request beyond
-// that pool would block forever; using the pool exactly is fine
-static_assert(kRegsIo + 2 * kRegsSoftmax <= 3 * 168, "registers traded between the warpgroups exceed the CTA's allocation");
+// registers per thread after the warpgroups have traded them (3 x 128 threads of 168 at launch, or 4 x 128 of 128)
+template <bool COPY> struct Regs { static constexpr int IO = COPY ? 112 : 104, SOFTMAX = COPY ? 168 : 200, TILES = 64; };
+// setmaxnreg only moves registers inside the CTA's own allocation: a request beyond that pool would block forever; using the
+// pool exactly is fine
+static_assert(Regs<false>::IO + 2 * Regs<false>::SOFTMAX <= 3 * 168, "registers traded between the warpgroups exceed the CTA's allocation");
+static_assert(Regs<true>::IO + 2 * Regs<true>::SOFTMAX + Regs<true>::TILES <= 4 * 128, "registers traded between the warpgroups exceed the CTA's allocation");
 constexpr int kRounds = 4;                 // a unit has at most 128 branches: 4 rounds of 32 lanes
-constexpr int kDescReaders = 5;            // readers of a pipeline's unit descriptor: its MMA thread and its four softmax warps
+template <bool COPY> constexpr int kDescReaders = COPY ? 7 : 5;     // of a pipeline's unit descriptor: MMA thread, four softmax warps, two copy warps
 constexpr int kMaxStages = 4;              // K or V stages of one pipeline (barrier storage)
 
 template <int D> struct Cfg {
@@ -72,7 +78,7 @@ template <int D> struct Cfg {
     static constexpr int OFF_K = OFF_STAGE + 8 * 2048;
     static constexpr int OFF_V = OFF_K + 2 * NK * KV_BYTES;
     static constexpr int OFF_MISC = OFF_V + 2 * NV * KV_BYTES;
-    static constexpr int SMEM = OFF_MISC + 4096;                 // + misc; the dynamic segment itself is 1024-B aligned
+    static constexpr int SMEM = OFF_MISC + 5120;                 // + misc; the dynamic segment itself is 1024-B aligned
     static_assert(NK <= kMaxStages && NV <= kMaxStages, "barrier storage");
 };
 static_assert(Cfg<128>::SMEM <= 232448, "shared memory budget");
@@ -108,13 +114,16 @@ struct UnitDesc {
     int kv_row0;     // first global prefix token row
     int blk_count;   // tokens of the block shared by several documents that precede this unit's prefix chunk (0: none)
     int blk_row0;    // first token row of that block in the block tensors
+    int nrounds;     // rounds of 32 branches whose cached tokens are packed
+    int pad[3];
     uint16_t cs[kM];     // per branch: packed column of its first cached token
     uint16_t len[kM];    // per branch: cached tokens visible (0 for a bad table entry)
     // position-order mode: the branches above are ALL slots of the group up to the unit's last row (live or retired);
     uint16_t ridx[kM];   // per row-branch of the unit: its index among them
     int32_t pvis[kM];    // per row-branch: prefix tokens of this unit's chunk it may see
+    int32_t off[kM];     // per branch (copy warps only): first row of its slab in the cache
 };
-static_assert(sizeof(UnitDesc) == 48 + 10 * kM, "descriptor size");
+static_assert(sizeof(UnitDesc) == 64 + 14 * kM, "descriptor size");
 
 struct Misc {
     unsigned long long q_full[2], q_empty[2];
@@ -127,7 +136,7 @@ struct Misc {
     UnitDesc desc[2];    // one per pipeline
 };
 
-static_assert(sizeof(Misc) <= 4096, "misc block");
+static_assert(sizeof(Misc) <= 5120, "misc block");
 
 // ------------------------------------------------------------------------------------------------
 // PTX wrappers
@@ -302,22 +311,32 @@ __device__ __forceinline__ void fill_tile(const Unit& u, int t, const int (&cs)[
 // ------------------------------------------------------------------------------------------------
 // the kernel
 // ------------------------------------------------------------------------------------------------
-// ORDER = false: branch-local mask (Eq. 5-6): a row sees its document's prefix and its own branch's cached tokens.
-// ORDER = true:  position-order mask (Sec. 4.3.2, Fig. 3): a group is a whole stacked prompt; a row sees the first
+// kOwn:          branch-local mask (Eq. 5-6): a row sees its document's prefix and its own branch's cached tokens.
+// kOrder:        position-order mask (Sec. 4.3.2, Fig. 3): a group is a whole stacked prompt; a row sees the first
 //                prefix_vis[row] prefix tokens (prompt and the skeleton up to its own attribute key) and the cached
 //                tokens of every slot of the group up to and including its own -- live or retired --, which is "position
 //                ID not larger than mine" under Algorithm 2's K_max gaps.  Branch tokens are packed back to back in slot
 //                order, so a row's visible packed columns are one range starting at 0.
-// BLOCK = true:  a third sharing level (Sec. 4.3.5): the documents' prefixes are preceded by a block of tokens common to
+// kPrefill:      the position-order mask over the prompts alone (Sec. 4.3.2, first inference step): rows are prompt tokens, no branch caches.
+// kBlock:        a third sharing level (Sec. 4.3.5): the documents' prefixes are preceded by a block of tokens common to
 //                several documents (instruction, attribute definitions), stored once in tensors of its own; a unit visits the
 //                block's tiles between its suffix tiles and its document's tiles.
-template <int D, bool ORDER, bool BLOCK>
-__global__ void __launch_bounds__(kThreads, 1)
+// Copy warps (position-order decode): a unit packs the cached tokens of up to 96 or 128 branches, each a copy of 1 to 16 rows per half of K
+//                and V, and a warp issues one about every 100 cycles.  One producer warp per pipeline was what the mode waited for (a
+//                tile of cached tokens took 5 k cycles, a prefix tile 1.1 k); with a warp for K and one for V besides the scheduler
+//                the attention of one prompt went 42.6 -> 31.1 us, of 64 prompts 360 -> 341.  The other modes pack a third of the
+//                branches and lose 1 to 5 % with sixteen warps, so they keep one warp for all of it.  Each ring has ONE producer, which
+//                waits through every phase of its barriers.
+template <int D, int MODE>
+__global__ void __launch_bounds__(kThreadsOf<MODE>, 1)
 hpd_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                    const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_bk,
                    const __grid_constant__ CUtensorMap map_bv, const __grid_constant__ SufMaps smaps, const TcParams p)
 {
     using C = Cfg<D>;
+    constexpr bool ORDER = MODE == kOrder || MODE == kPrefill, BLOCK = MODE == kBlock, COPY = kCopyWarps<MODE>;
+    constexpr int kThreads = kThreadsOf<MODE>;
+    using R = Regs<COPY>;
     extern __shared__ __align__(1024) uint8_t smem[];
     Misc* misc = reinterpret_cast<Misc*>(smem + C::OFF_MISC);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -333,7 +352,7 @@ hpd_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             mbar_init(&misc->q_full[i], 1);  mbar_init(&misc->q_empty[i], 1);
             for (int b = 0; b < 2; ++b) { mbar_init(&misc->s_full[i][b], 1); mbar_init(&misc->p_full[i][b], 4); mbar_init(&misc->p_empty[i][b], 1); }
             mbar_init(&misc->o_full[i], 1);  mbar_init(&misc->o_free[i], 4);
-            mbar_init(&misc->desc_full[i], 1); mbar_init(&misc->desc_empty[i], kDescReaders);
+            mbar_init(&misc->desc_full[i], 1); mbar_init(&misc->desc_empty[i], kDescReaders<COPY>);
             for (int k = 0; k < kMaxStages; ++k) {
                 mbar_init(&misc->k_full[i][k], 1); mbar_init(&misc->k_empty[i][k], 1);
                 mbar_init(&misc->v_full[i][k], 1); mbar_init(&misc->v_empty[i][k], 1);
@@ -363,7 +382,7 @@ hpd_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         // consumed an iteration after it was issued: ticket (i+4) -> work item (i+3) -> document tables (i+2) ->
         // branch table (i+1) -> scan, publish and produce the tiles (i).  (An iteration lasts a whole unit, ten
         // microseconds or more, so one stage per iteration is ample for an L2 round trip.)
-        reg_dealloc<kRegsIo>();
+        reg_dealloc<R::IO>();
         const int x = warp == 0 ? 0 : 1;
         const int Hkv = p.a.g.Hkv;
         // The pipeline's first unit is one of two, whichever way the units are laid over the SMs: both items are asked for together with
@@ -420,7 +439,7 @@ hpd_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         }
         // position-order mode: first slot of the group and of the next one
         int dss1 = 0, dse1 = 0, dss0 = 0, dse0 = 0;
-        const bool have_slots = ORDER && p.a.slot_depth != nullptr;      // false: no branch cache at all (the prefill)
+        constexpr bool have_slots = MODE == kOrder;      // false: no branch cache at all (the prefill)
         if (have_slots) {
             dss1 = p.a.doc_slot_start[it1.doc]; dse1 = p.a.doc_slot_start[it1.doc + 1];
             dss0 = p.a.doc_slot_start[it0.doc]; dse0 = p.a.doc_slot_start[it0.doc + 1];
@@ -519,6 +538,7 @@ hpd_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 cs[r] = carry + incl - n; len[r] = n; off[r] = o;
                 d.cs[b] = static_cast<uint16_t>(cs[r]);
                 d.len[b] = static_cast<uint16_t>(n);
+                if constexpr (COPY) d.off[b] = o;
                 carry += __shfl_sync(0xffffffffu, incl, 31);
             }
             if (__any_sync(0xffffffffu, bad) && lane == 0 && p.a.dev_status) atomicOr(p.a.dev_status, HPD_S_BAD_TABLE);
@@ -534,13 +554,26 @@ hpd_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             if (lane == 0) {
                 d.nt = u.nt; d.np = u.np; d.stot = u.stot; d.head = u.head; d.key_count = u.key_count; d.part_base = u.part_base;
                 d.row_begin = u.row_begin; d.nb = u.nb; d.row0 = u.row0; d.kv_row0 = u.kv_row0;
-                d.blk_count = u.blk_count; d.blk_row0 = u.blk_row0;
+                d.blk_count = u.blk_count; d.blk_row0 = u.blk_row0; d.nrounds = nrounds;
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(&misc->desc_full[x]);
             if (!live) break;
-            // ---- the unit's tiles: K runs one tile ahead of V, the order in which the MMA warp consumes them ----
+            auto fetch_q = [&]() {
+                ok = mbar_wait_warp(&misc->q_empty[x], (qc & 1) ^ 1, misc);
+                if (ok && lane == 0) {
+                    mbar_expect_tx(&misc->q_full[x], C::Q_BYTES);
+                    for (int h = 0; h < C::HALVES; ++h)
+                        tma_load_4d(q_tile + h * kQHalf, &map_q, &misc->q_full[x], h * 64, 0, u.head, u.row0);
+                }
+                ++qc;
+            };
             const int nt = u.nt;
+            if constexpr (COPY) {
+                if (nt > 0) fetch_q();
+                __syncwarp();
+            } else {
+            // ---- the unit's tiles: K runs one tile ahead of V, the order in which the MMA warp consumes them ----
             for (int t = 0; t <= nt && ok; ++t) {
                 if (t < nt) {
                     const int ks = kc % C::NK;
@@ -548,18 +581,10 @@ hpd_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                     if (!ok) break;
                     fill_tile<D>(u, t, cs, len, off, nrounds, lane, k_ring + ks * C::KV_BYTES, &misc->k_full[x][ks], &map_k, &map_bk, smaps.k);
                     ++kc;
-                    if (t == 0) {
-                        // The Q tile is asked for after the unit's first K tile: its buffer is released late in the
-                        // previous unit, and waiting for it first would hold up the tile that can be fetched already.
-                        ok = mbar_wait_warp(&misc->q_empty[x], (qc & 1) ^ 1, misc);
-                        if (!ok) break;
-                        if (lane == 0) {
-                            mbar_expect_tx(&misc->q_full[x], C::Q_BYTES);
-                            for (int h = 0; h < C::HALVES; ++h)
-                                tma_load_4d(q_tile + h * kQHalf, &map_q, &misc->q_full[x], h * 64, 0, u.head, u.row0);
-                        }
-                        ++qc;
-                    }
+                    // The Q tile is asked for after the unit's first K tile: its buffer is released late in the
+                    // previous unit, and waiting for it first would hold up the tile that can be fetched already.
+                    if (t == 0) fetch_q();
+                    if (!ok) break;
                 }
                 if (t >= 1) {
                     const int vs = vc % C::NV;
@@ -569,6 +594,7 @@ hpd_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                     ++vc;
                 }
                 __syncwarp();
+            }
             }
             // ---- shift the pipeline ----
             w0 = w1; w1 = w2; w2 = w3; w3 = w4;
@@ -585,7 +611,7 @@ hpd_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         }
     } else if (warp < 3) {
         // ================================ MMA issuers (one per pipeline) =============================
-        reg_dealloc<kRegsIo>();
+        reg_dealloc<R::IO>();
         if (elect_one()) {
             const int x = warp - 1;
             uint32_t qc = 0, tiles = 0;                   // units with tiles so far; tiles of earlier units
@@ -669,9 +695,39 @@ hpd_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 tiles += nt;
             }
         }
+    } else if (COPY && warp >= 12) {
+        // ======================= TMA producers: the K tiles or the V tiles of one pipeline ===================
+        reg_dealloc<R::TILES>();
+        const int x = (warp - 12) >> 1, is_v = warp & 1;
+        const uint32_t stages = is_v ? C::NV : C::NK;
+        uint8_t* ring = smem + (is_v ? C::OFF_V + x * C::NV * C::KV_BYTES : C::OFF_K + x * C::NK * C::KV_BYTES);
+        unsigned long long *full = is_v ? misc->v_full[x] : misc->k_full[x], *empty = is_v ? misc->v_empty[x] : misc->k_empty[x];
+        const CUtensorMap *pre = is_v ? &map_v : &map_k, *suf = is_v ? smaps.v : smaps.k;
+        const UnitDesc& d = misc->desc[x];
+        uint32_t c = 0;                                  // tiles so far
+        bool ok = true;
+        for (uint32_t ui = 0; ok; ++ui) {
+            ok = mbar_wait_warp(&misc->desc_full[x], ui & 1, misc);
+            if (!ok) break;
+            Unit u = read_unit(d);
+            const int nrounds = d.nrounds;
+            int cs[kRounds], len[kRounds], off[kRounds];
+#pragma unroll
+            for (int r = 0; r < kRounds; ++r) { cs[r] = d.cs[lane + 32 * r]; len[r] = d.len[lane + 32 * r]; off[r] = d.off[lane + 32 * r]; }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&misc->desc_empty[x]);
+            if (u.nt < 0) break;
+            for (int t = 0; t < u.nt; ++t, ++c) {
+                const uint32_t st = c % stages;
+                ok = mbar_wait_warp(&empty[st], ((c / stages) & 1) ^ 1, misc);
+                if (!ok) break;
+                fill_tile<D>(u, t, cs, len, off, nrounds, lane, ring + st * C::KV_BYTES, &full[st], pre, pre, suf);
+                __syncwarp();
+            }
+        }
     } else {
         // ======================================= softmax A / B =======================================
-        reg_alloc<kRegsSoftmax>();
+        reg_alloc<R::SOFTMAX>();
         const int x = warp >= 8 ? 1 : 0;                 // pipeline
         const int quad = warp & 3;                       // TMEM lane quadrant this warp may access
         const int row = quad * 32 + lane;                // tile row = TMEM lane
@@ -1039,7 +1095,7 @@ bool make_q_map(CUtensorMap* m, const void* base, int D, int G, int Hkv, long lo
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int D, bool ORDER, bool BLOCK>
+template <int D, int MODE>
 int launch_d(const AttnArgs& a)
 {
     using C = Cfg<D>;
@@ -1047,7 +1103,7 @@ int launch_d(const AttnArgs& a)
     static std::atomic<bool> attr_set[kMaxDevices];
     const int dev = current_device();
     if (dev < 0 || dev >= kMaxDevices || !attr_set[dev].load(std::memory_order_acquire)) {
-        HPD_CUDA_TRY(cudaFuncSetAttribute(hpd_attn_tc_kernel<D, ORDER, BLOCK>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
+        HPD_CUDA_TRY(cudaFuncSetAttribute(hpd_attn_tc_kernel<D, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
         if (dev >= 0 && dev < kMaxDevices) attr_set[dev].store(true, std::memory_order_release);
     }
     const int G = a.g.Hq / a.g.Hkv;
@@ -1100,13 +1156,13 @@ int launch_d(const AttnArgs& a)
     p.G = G;
     const int n_sm = sm_count();
     CUtensorMap mbk = mk, mbv = mv;                      // unused without a shared block
-    if constexpr (BLOCK) {
+    if constexpr (MODE == kBlock) {
         if (!make_kv_map(&mbk, a.block_k, D, a.g.Hkv, a.total_block, kN) || !make_kv_map(&mbv, a.block_v, D, a.g.Hkv, a.total_block, kN)) {
             set_last_cuda_error(cudaErrorInvalidValue);
             return HPD_E_CUDA;
         }
     }
-    HPD_CUDA_TRY(launch_chained(hpd_attn_tc_kernel<D, ORDER, BLOCK>, n_sm, kThreads, C::SMEM, a.stream, mq, mk, mv, mbk, mbv, sm, p));
+    HPD_CUDA_TRY(launch_chained(hpd_attn_tc_kernel<D, MODE>, n_sm, kThreadsOf<MODE>, C::SMEM, a.stream, mq, mk, mv, mbk, mbv, sm, p));
     // one warp per (row, q head) where the rows allow it, at most one resident wave; with many documents nothing is
     // split as a rule (the kernel then only rewinds the ticket counter) and a small grid is launched sooner
     const long long merge_blocks = (static_cast<long long>(a.max_rows) * a.g.Hq + 7) / 8;
@@ -1121,9 +1177,11 @@ int launch_d(const AttnArgs& a)
 int launch_attn_tc(const AttnArgs& a)
 {
     if (!(a.g.sm_scale > 0.f)) return HPD_E_GEOM;
-    if (a.prefix_vis) return a.g.D == 128 ? launch_d<128, true, false>(a) : launch_d<64, true, false>(a);
-    if (a.block_k) return a.g.D == 128 ? launch_d<128, false, true>(a) : launch_d<64, false, true>(a);
-    return a.g.D == 128 ? launch_d<128, false, false>(a) : launch_d<64, false, false>(a);
+    const bool wide = a.g.D == 128;
+    if (a.prefix_vis && a.slot_depth) return wide ? launch_d<128, kOrder>(a) : launch_d<64, kOrder>(a);
+    if (a.prefix_vis) return wide ? launch_d<128, kPrefill>(a) : launch_d<64, kPrefill>(a);
+    if (a.block_k) return wide ? launch_d<128, kBlock>(a) : launch_d<64, kBlock>(a);
+    return wide ? launch_d<128, kOwn>(a) : launch_d<64, kOwn>(a);
 }
 
 }  // namespace hpd
