@@ -232,6 +232,31 @@ __device__ __forceinline__ void rank_keys(uint32_t* key, int n2, int n_items, ui
     __syncthreads();
 }
 
+// The same by counting, for short lists: a key's place is the number of smaller ones.  1024 / n2 threads share a key and compare it with
+// an equal part of the others (n2^2 / 1024 comparisons a thread, read four at a time by all lanes of a warp alike), so nothing
+// waits for anything but two barriers, where the bitonic network is 21 to 45 dependent stages.
+// key: n2 keys (a power of two, 64 to kCountItems), key[w] being that of item w; cnt: n2 counters.
+constexpr int kCountItems = 512;
+
+__device__ __forceinline__ void count_ranks(const uint32_t* key, int n2, int n_items, uint32_t* cnt, uint16_t* rank)
+{
+    const int t = threadIdx.x, i = t & (n2 - 1), part = t / n2, len = n2 * n2 / kPlanThreads;
+    if (t < n2) cnt[t] = 0;
+    __syncthreads();
+    const uint32_t mine = key[i];
+    const uint4* other = reinterpret_cast<const uint4*>(key + part * len);
+    uint32_t smaller = 0;
+#pragma unroll 4
+    for (int j = 0; j < len / 4; ++j) {
+        const uint4 k = other[j];
+        smaller += (k.x < mine) + (k.y < mine) + (k.z < mine) + (k.w < mine);
+    }
+    atomicAdd(&cnt[i], smaller);
+    __syncthreads();
+    if (t < n_items) rank[t] = static_cast<uint16_t>(cnt[t]);
+    __syncthreads();
+}
+
 // Block-wide exclusive scan of one 64-bit word per thread (two packed ints) by 1024 threads behind ONE barrier: every warp
 // scans the 32 warp totals for itself.  buf alternates between consecutive calls.
 __device__ __forceinline__ long long scan_words(long long v, long long* buf, long long& total)
@@ -369,11 +394,12 @@ __device__ __forceinline__ void plan_block(int n_docs, int G, int Hkv, int n_sm,
         }
         if (n_items > 1 && n_items <= kSortItems) {
             sorted = true;
-            int n2 = 2;
+            int n2 = 64;
             while (n2 < n_items) n2 <<= 1;
             for (int w = n_items + threadIdx.x; w < n2; w += kPlanThreads) s_key[w] = 0xFFFFFFFFu;
             __syncthreads();
-            rank_keys(s_key, n2, n_items, rank);
+            if (n2 <= kCountItems) count_ranks(s_key, n2, n_items, s_key + kCountItems, rank);
+            else rank_keys(s_key, n2, n_items, rank);
         }
     }
 
@@ -451,7 +477,7 @@ plan_kernel(int n_docs, int n_slots, int G, int Hkv, int n_sm,
         }
         return;
     }
-    __shared__ int s_scratch[kPlanScratchInts];
+    __shared__ __align__(16) int s_scratch[kPlanScratchInts];
     __shared__ uint16_t s_rank[kSortItems];
     plan_block(n_docs, G, Hkv, n_sm, doc_prefix_len, doc_active_start, s_scratch, s_rank,
                              hdr, work, split, work_cap, part_cap);
@@ -492,7 +518,7 @@ meta_step_kernel(int n_docs, int n_slots, int32_t suffix_cap, int32_t pos_gap, i
 {
     __shared__ int s_start[kStepDocs + 1];           // first slot of every document; block 0 turns it into its first row
     __shared__ int s_len[kStepDocs];
-    __shared__ uint32_t s_bits[kStepWords + kStepWords / 2];      // live mask, then the 16-bit prefix counts
+    __shared__ __align__(16) uint32_t s_bits[kStepWords + kStepWords / 2];      // live mask, then the 16-bit prefix counts
     __shared__ long long s_scan[2][32];
     __shared__ int s_cnt[32];
     uint32_t* s_mask = s_bits;
