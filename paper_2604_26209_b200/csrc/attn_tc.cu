@@ -277,7 +277,7 @@ __device__ __forceinline__ void fill_tile(const Unit& u, int t, const int (&cs)[
     const int nbt = block_tiles(u);
     const int ns = u.nt - u.np - nbt;
     if (t >= ns) {
-        if (lane == 0) {
+        if (elect_one()) {
             mbar_expect_tx(full, C::KV_BYTES);
             const bool in_block = t - ns < nbt;
             const CUtensorMap* m = in_block ? blk : pre;
@@ -561,7 +561,7 @@ hpd_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             if (!live) break;
             auto fetch_q = [&]() {
                 ok = mbar_wait_warp(&misc->q_empty[x], (qc & 1) ^ 1, misc);
-                if (ok && lane == 0) {
+                if (ok && elect_one()) {
                     mbar_expect_tx(&misc->q_full[x], C::Q_BYTES);
                     for (int h = 0; h < C::HALVES; ++h)
                         tma_load_4d(q_tile + h * kQHalf, &map_q, &misc->q_full[x], h * 64, 0, u.head, u.row0);
