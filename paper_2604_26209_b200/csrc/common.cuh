@@ -71,7 +71,8 @@ static_assert(sizeof(WsHeader) == 128, "header size");
 // with_suffix is set.  part_base < 0: the item produces the final output of its rows.
 struct WorkItem {
     int32_t doc, key_begin, key_count, part_base;
-    int32_t row_begin, row_count, with_suffix, pad;
+    int32_t row_begin, row_count, with_suffix;
+    int32_t doc_row;                 // first row of the document
 };
 static_assert(sizeof(WorkItem) == 32, "work item size");
 
@@ -157,8 +158,8 @@ int launch_attn_tc(const AttnArgs& a);       // tcgen05 / TMA kernel
 // Launches that may start while their predecessor in the stream ends.  The kernel is scheduled as soon as every block of the
 // predecessor has called start_dependents() (or has ended), does what needs no memory of others, and calls
 // await_predecessors() before its first access to global memory; that returns once the predecessor has completed and its
-// writes are visible.  Every kernel launched like this waits in all of its blocks, so "the predecessor has completed"
-// includes everything before it.
+// writes are visible.  Every kernel launched like this waits in all of its blocks, or in at least one of them where the others touch
+// nothing (the merge kernel), so "the predecessor has completed" includes everything before it.
 // Such a kernel is resident while others still write what it will read: none of its pointer parameters is __restrict__, which would
 // promise that nothing else writes there during the kernel's life and so allow reads through the non-coherent path or above the wait.
 // ---------------------------------------------------------------------------------------------
@@ -166,10 +167,10 @@ __device__ __forceinline__ void await_predecessors() { asm volatile("griddepcont
 __device__ __forceinline__ void start_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <typename... P, typename... A>
-cudaError_t launch_chained(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t stream, A&&... args)
+cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t stream, A&&... args)
 {
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(grid); cfg.blockDim = dim3(block); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
+    cfg.gridDim = grid; cfg.blockDim = dim3(block); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
     cudaLaunchAttribute attr{};
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;

@@ -436,7 +436,7 @@ __device__ __forceinline__ void plan_block(int n_docs, int G, int Hkv, int n_sm,
                     it.row_count = min(rows_per_block, rows - it.row_begin);
                     it.part_base = ch > 1 ? ep + c * rows : -1;
                     it.with_suffix = (c == ch - 1);
-                    it.pad = 0;
+                    it.doc_row = doc_active_start[d];
                     work[sorted ? static_cast<int>(rank[w]) : w] = it;
                 }
             }
@@ -733,7 +733,7 @@ prefill_meta_kernel(int n_docs, int G, int32_t pos_gap,
         WorkItem it;
         it.doc = d; it.key_begin = 0; it.key_count = min(L, (m + 1) * rpb);
         it.part_base = -1; it.row_begin = m * rpb; it.row_count = min(rpb, L - m * rpb);
-        it.with_suffix = 0; it.pad = 0;
+        it.with_suffix = 0; it.doc_row = s_kv[d];
         work[x] = it;
     }
     if (blockIdx.x == 0) {
