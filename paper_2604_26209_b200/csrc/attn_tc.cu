@@ -34,18 +34,19 @@
 #include <atomic>
 
 #include "common.cuh"
+#include "copy_warps.h"
 #include "ptx.cuh"
 
 namespace hpd {
 
 namespace {
 
-// What a launch attends (template parameter): own document and branch (kOwnFew: in steps of few units); the same with a block shared by
+// What a launch attends (template parameter): own document and branch (kOwnCopy: in steps that copy_warps.h picks); the same with a block shared by
 // several documents in front; position-order mask over a group's prefix and branch caches; position-order mask over prompts alone
 // (first inference step).
-enum Mode { kOwn, kOwnFew, kBlock, kOrder, kPrefill };
-// The position-order decode and steps of few units have four more warps, which copy K and V tiles (the reason stands at the kernel).
-template <int MODE> constexpr bool kCopyWarps = MODE == kOrder || MODE == kOwnFew;
+enum Mode { kOwn, kOwnCopy, kBlock, kOrder, kPrefill };
+// The position-order decode and those steps have four more warps, which copy K and V tiles (the reason stands at the kernel).
+template <int MODE> constexpr bool kCopyWarps = MODE == kOrder || MODE == kOwnCopy;
 template <int MODE> constexpr int kThreadsOf = kCopyWarps<MODE> ? 512 : 384;
 constexpr int kM = 128;                    // rows of a tile
 constexpr int kN = 64;                     // keys of a tile
@@ -326,10 +327,11 @@ __device__ __forceinline__ void fill_tile(const Unit& u, int t, const int (&cs)[
 //                rows per half of D and of K and V, and a warp issues one about every 100 cycles.  One producer warp per pipeline was what
 //                the position-order decode waited for (a tile of cached tokens took 5 k cycles, a prefix tile 1.1 k); with a warp for K and
 //                one for V besides the scheduler the attention of one prompt went 42.6 -> 30.9 us, of 64 prompts 358 -> 336.  Steps of
-//                few units wait for the same copies before anything else (kOwnFew; one prompt 18.8 -> 17.6 us, with the second pipeline's
-//                idle warps helping; the position-order mask there 30.5 -> 28.5).  The other launches pack fewer branches on pipelines
-//                that hide the copies behind each other, and lose 1 to 5 % with sixteen warps, so they keep one warp for all
-//                of it.  Each ring has ONE producer (or a pair that both wait through every phase of its barriers).
+//                few units of many branches wait for the same copies before anything else (kOwnCopy; one prompt 18.8 -> 17.6 us, with
+//                the second pipeline's idle warps helping; the position-order mask there 30.5 -> 28.5).  The other launches pack fewer
+//                branches on pipelines that hide the copies behind each other, and lose 1 to 8 % with sixteen warps, so they keep one
+//                warp for all of it (the line: copy_warps.h).  Each ring has ONE producer (or a pair that both wait through every phase of
+//                its barriers).
 template <int D, int MODE>
 __global__ void __launch_bounds__(kThreadsOf<MODE>, 1)
 hpd_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
@@ -1200,9 +1202,9 @@ int launch_attn_tc(const AttnArgs& a)
     const bool wide = a.g.D == 128;
     if (a.prefix_vis && a.slot_depth) return wide ? launch_d<128, kOrder>(a) : launch_d<64, kOrder>(a);
     if (a.prefix_vis) return wide ? launch_d<128, kPrefill>(a) : launch_d<64, kPrefill>(a);
-    // few units: at most one on an SM when none is split and none has several row blocks
-    if (!a.block_k && static_cast<long long>(a.n_docs) * a.g.Hkv <= sm_count()) return wide ? launch_d<128, kOwnFew>(a) : launch_d<64, kOwnFew>(a);
     if (a.block_k) return wide ? launch_d<128, kBlock>(a) : launch_d<64, kBlock>(a);
+    if (copy_warps_pay({a.n_docs, a.max_rows, a.total_prefix, a.g.Hq / a.g.Hkv, a.g.Hkv, a.g.D, sm_count(), a.lay.work_cap, a.lay.part_cap}))
+        return wide ? launch_d<128, kOwnCopy>(a) : launch_d<64, kOwnCopy>(a);
     return wide ? launch_d<128, kOwn>(a) : launch_d<64, kOwn>(a);
 }
 

@@ -27,3 +27,26 @@ def oracle_step(s, t_bits, n_threads=0, rows=None):
 def err_stats(got, want):
     d = np.abs(np.asarray(got, dtype=np.float64) - np.asarray(want, dtype=np.float64))
     return (float(d.max()) if d.size else 0.0, float(d.mean()) if d.size else 0.0)
+
+
+def copy_warps_rule(build_dir):
+    """The host rule that picks a decode launch's kernel, compiled from its header: f(n_docs, max_rows, total_prefix, G, Hkv, D, n_sm, work_cap,
+    part_cap) -> (copy warps, expected units)."""
+    import ctypes
+    import os
+    import subprocess
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    src, lib = os.path.join(build_dir, "rule.cpp"), os.path.join(build_dir, "rule.so")
+    with open(src, "w") as f:
+        f.write('#include "copy_warps.h"\nextern "C" long long rule(const hpd::StepSize* s, int* pay)\n'
+                "{ *pay = hpd::copy_warps_pay(*s); return hpd::average_unit(*s).units; }\n")
+    subprocess.run(["g++", "-O1", "-std=c++17", "-Wall", "-Werror", "-shared", "-fPIC", "-I", os.path.join(root, "paper_2604_26209_b200", "csrc"), src,
+                    "-o", lib], check=True)
+    fn = ctypes.CDLL(lib).rule
+    fn.restype = ctypes.c_longlong
+
+    def call(*sizes):
+        pay = ctypes.c_int()
+        units = fn((ctypes.c_int * 9)(*sizes), ctypes.byref(pay))
+        return bool(pay.value), units
+    return call
