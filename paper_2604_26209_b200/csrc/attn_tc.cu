@@ -388,10 +388,10 @@ hpd_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         // document and branch tables (i+1) -> scan, publish and produce the tiles (i).  (An iteration lasts a whole unit, ten
         // microseconds or more, so one stage per iteration is ample for an L2 round trip.)  Nothing precedes the first unit, so its
         // loads are all that is asked for before it is published: two round trips, the work item and then its tables, because the item
-        // carries its document's first row (checked against the table, which has the last word).  Later units' loads follow the
-        // unit's first K tile.  With four round trips and the other units' loads among them the first copy of a launch began 3.7 k
-        // cycles after its predecessor had ended, now 3.1 k (attention call of 8 prompts 25.2 -> 24.8 us, first inference step of one
-        // prompt 50.8 -> 49.8).
+        // carries its document's first row (checked against the table, which has the last word).  Later units' loads stand at the
+        // unit's Q tile, before or behind it (see there).  With four round trips and the other units' loads among them the first copy of a
+        // launch began 3.7 k cycles after its predecessor had ended, now 3.1 k (attention call of 8 prompts 25.2 -> 24.8 us, first
+        // inference step of one prompt 50.8 -> 49.8).
         reg_dealloc<R::IO>();
         const int x = warp == 0 ? 0 : 1;
         const int Hkv = p.a.g.Hkv;
@@ -587,6 +587,11 @@ hpd_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 if (nt > 0 && ui > 0) fetch_q();
                 __syncwarp();
             } else {
+            // With four stages to a ring the producer is ahead of the MMA warp until it waits for Q, and what it does behind that wait holds up
+            // the unit's next tiles: the next units' loads then belong in front of it (600 documents of 512 tokens at D = 64: 24 branches
+            // 156 -> 153 us a step, 48 branches 218 -> 214).  With two stages it never is ahead, and Q has to come first (D = 128,
+            // 64 documents 59.8 against 61.0 us); the shared block and the first step measured equal or 1 % better like that at both D.
+            constexpr bool kBeforeQ = MODE == kOwn && C::NK > 2;
             // ---- the unit's tiles: K runs one tile ahead of V, the order in which the MMA warp consumes them ----
             for (int t = 0; t <= nt && ok; ++t) {
                 if (t < nt) {
@@ -597,10 +602,14 @@ hpd_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                     ++kc;
                     // The Q tile is asked for after the unit's first K tile: its buffer is released late in the
                     // previous unit, and waiting for it first would hold up the tile that can be fetched already.
-                    if (t == 0) fetch_q();
+                    if (t == 0 && !(kBeforeQ && ui > 0)) fetch_q();
                     if (!ok) break;
                 }
-                if (t == 0) next_stage();
+                if (t == 0) {
+                    next_stage();
+                    if (kBeforeQ && ui > 0 && nt > 0) fetch_q();
+                    if (!ok) break;
+                }
                 if (t >= 1) {
                     const int vs = vc % C::NV;
                     ok = mbar_wait_warp(&misc->v_empty[x][vs], ((vc / C::NV) & 1) ^ 1, misc);
