@@ -16,8 +16,10 @@
  *   - every call only ENQUEUES work on `stream` (a cudaStream_t passed as void*) and never
  *     synchronises.  Sizes that change per step (n_active) are read on the device.
  *   - kernels are launched chained (programmatic stream serialisation): one may be resident before its
- *     predecessor in the stream has ended, and waits for it before it touches device memory.  Ordinary
- *     launches, copies and events around the calls are ordered as always.  A caller's own kernel that is launched
+ *     predecessor in the stream has ended, and waits for it before it touches device memory (inside an
+ *     attention call the second kernel looks at the call's work list before it waits; the first lets it in
+ *     only after its own wait, so whatever wrote that list has ended).  Ordinary launches, copies and
+ *     events around the calls are ordered as always.  A caller's own kernel that is launched
  *     programmatically BEHIND a call may start before that call has ended: it has to wait
  *     (cudaGridDependencySynchronize) before it touches anything that this or an earlier call in the
  *     stream reads or writes.  One IN FRONT of a call has to wait in all of its blocks, too: a call
