@@ -17,8 +17,9 @@
 // tiles and an output accumulator (tensor memory), and these warps:
 //
 //   warp 0 / 3    scheduler and TMA producer: draws the pipeline's units, publishes their
-//                 descriptors, issues Q, K and V tiles (prefix: lane 0; suffix boxes: all lanes);
-//                 in the position-order decode warps 12 / 14 issue the K tiles and 13 / 15 the V tiles
+//                 descriptors, issues Q, K and V tiles (Q and prefix: an elected lane; suffix boxes: all
+//                 lanes); in launches with copy warps (position-order decode, and the steps that
+//                 copy_warps.h picks) warps 12 / 14 issue the K tiles and 13 / 15 the V tiles
 //   warp 1 / 2    MMA issuer: S = Q K^T (both operands in shared memory), two tiles ahead of the
 //                 softmax, and O += P V (P in tensor memory, V in shared memory); tcgen05.mma
 //   warps 4-7 /   softmax: one thread per row: S from TMEM, online max/sum, P as bf16 pairs written
@@ -263,7 +264,7 @@ __device__ __forceinline__ Unit read_unit(const UnitDesc& d) {
     return u;
 }
 
-// One K or V tile of a unit.  A prefix tile is two boxes issued by lane 0; a suffix tile is packed from one box per
+// One K or V tile of a unit.  A prefix tile is a box per half of D issued by an elected lane; a suffix tile is packed from one box per
 // branch (and half), every lane placing the part of its branches that falls into the tile.  Boxes have the exact height
 // of the piece (tensor maps for 1..16 rows), so nothing beyond a branch's length is ever read: whatever lies there in
 // the cache -- possibly NaN -- must not meet a zero probability, and the packing needs no padding.
@@ -331,7 +332,8 @@ __device__ __forceinline__ void fill_tile(const Unit& u, int t, const int (&cs)[
 //                the second pipeline's idle warps helping; the position-order mask there 30.5 -> 28.5).  The other launches pack fewer
 //                branches on pipelines that hide the copies behind each other, and lose 1 to 8 % with sixteen warps, so they keep one
 //                warp for all of it (the line: copy_warps.h).  Each ring has ONE producer (or a pair that both wait through every phase of
-//                its barriers).
+//                its barriers).  At 128 registers a thread these forms spill a little at D = 128 (kOwnCopy 20 bytes stored and 44 loaded,
+//                kOrder 16 and 16; in which role is not known), the others nothing.
 template <int D, int MODE>
 __global__ void __launch_bounds__(kThreadsOf<MODE>, 1)
 hpd_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
@@ -1193,8 +1195,8 @@ int launch_d(const AttnArgs& a)
         }
     }
     HPD_CUDA_TRY(launch_chained(hpd_attn_tc_kernel<D, MODE>, n_sm, kThreadsOf<MODE>, C::SMEM, a.stream, mq, mk, mv, mbk, mbv, sm, p));
-    // one warp per (row, q head) where the rows allow it, at most one resident wave; with many documents nothing is
-    // split as a rule (the kernel then only rewinds the ticket counter) and a small grid is launched sooner
+    // one warp per (row, q head) where the rows allow it, at most two resident waves (four blocks an SM); with many documents
+    // nothing is split as a rule (the kernel then only rewinds the ticket counter) and a small grid is launched sooner
     const long long merge_blocks = (static_cast<long long>(a.max_rows) * a.g.Hq + 7) / 8;
     const long long merge_cap = static_cast<long long>(a.n_docs) * a.g.Hkv < 4ll * n_sm ? 8ll * n_sm : 2ll * n_sm;
     const int merge_grid = MODE == kPrefill ? 1          // never split

@@ -20,8 +20,8 @@ template <bool FUSED> constexpr int kRopeResident = FUSED ? 6 : 8;   // CTAs of 
 // HBM bound: 26 KB a row, 24.4 us at the copy rate for 6144 rows; measured 28 us.  One CTA per two rows of 128 threads: with four rows
 // and 256 threads the last wave of 64 prompts was a third full and small steps had fewer CTAs than SMs (8 prompts 38.0 -> 37.5 us
 // a step, 32 prompts 108.2 -> 107.3, the first inference step of 64 prompts, rotation only, 3.35 -> 3.33 ms).  The rotation
-// alone is held to 64 registers, eight CTAs per SM (1 prompt's first inference step 64.4 -> 62.6 us); the fused kernel spills
-// nothing at 80 and lost 5 to 8 % of the step at 64.
+// alone is held to 64 registers, eight CTAs per SM (1 prompt's first inference step 64.4 -> 62.6 us); the fused kernel has 80
+// and lost 5 to 8 % of the step at 64.  Neither spills; their shared forms (below) spill 8 bytes fused and 28 alone.
 // Every thread first asks for its share of the rows' q / k / v chunks (up to ten 16-byte loads in
 // flight per thread), then evaluates one of the rows' D/2 (cos, sin) pairs; they are kept in shared memory as fp32 and
 // applied to all Hq + Hkv heads: a thread rotates 8 pairs at a time from one 16-byte chunk of the low half and one of the high half.
