@@ -1214,7 +1214,7 @@ int launch_attn_tc(const AttnArgs& a)
     if (a.prefix_vis && a.slot_depth) return wide ? launch_d<128, kOrder>(a) : launch_d<64, kOrder>(a);
     if (a.prefix_vis) return wide ? launch_d<128, kPrefill>(a) : launch_d<64, kPrefill>(a);
     if (a.block_k) return wide ? launch_d<128, kBlock>(a) : launch_d<64, kBlock>(a);
-    if (copy_warps_pay({a.n_docs, a.max_rows, a.total_prefix, a.g.Hq / a.g.Hkv, a.g.Hkv, a.g.D, sm_count(), a.lay.work_cap, a.lay.part_cap}))
+    if (copy_warps_pay({a.n_docs, a.max_rows, a.total_prefix, a.g.Hq / a.g.Hkv, a.g.Hkv, a.g.D, sm_count(), a.lay.work_cap, a.lay.part_cap, a.suffix_extra}))
         return wide ? launch_d<128, kOwnCopy>(a) : launch_d<64, kOwnCopy>(a);
     return wide ? launch_d<128, kOwn>(a) : launch_d<64, kOwn>(a);
 }

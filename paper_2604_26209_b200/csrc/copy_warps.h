@@ -9,6 +9,7 @@ struct StepSize {
     int n_docs, max_rows, total_prefix;
     int G, Hkv, D;
     int n_sm, work_cap, part_cap;    // SMs; work items and partial rows that the workspace holds
+    int new_tokens;                  // every branch has a cached token: the call sees those of this step
 };
 struct AverageUnit { long long units; int branches, keys; };
 
@@ -38,9 +39,11 @@ inline AverageUnit average_unit(const StepSize& s)
 //     The line lies at 13 keys a branch, 20 at D = 64 (52 branches and 1024 keys), and 96 branches take them always;
 //   four units an SM and more: short units of 32 branches gain a little too (960 units, 128 keys 54.5 / 56.1, a step 76.8 / 80.2, 512 keys 100.6 /
 //     103.1, 2048 keys 202 / 198; but 480 units of 128 keys 32.8 / 31.1).
+//   A call that does not see the step's tokens is as a rule one over a block's rows without branch caches: nothing to pack (6144 rows over
+//     128 tokens 42.2 / 36.3, 96 rows 10.0 / 8.8), so it never takes them.
 inline bool copy_warps_pay(const StepSize& s)
 {
-    if (static_cast<long long>(s.n_docs) * s.Hkv > s.n_sm) return false;
+    if (!s.new_tokens || static_cast<long long>(s.n_docs) * s.Hkv > s.n_sm) return false;
     const AverageUnit u = average_unit(s);
     if (u.units <= s.n_sm) return u.branches >= 22;
     if (u.units >= 4ll * s.n_sm && u.branches >= 32 && u.keys <= 16 * u.branches) return true;

@@ -44,3 +44,10 @@ def test_largest_sizes_do_not_overflow(rule):
     big = 2 ** 31 - 1
     assert rule(1, big, big, 1, 1, 128, SM, big, big)[1] == (big - 1) // 128 + 1
     assert rule(big, big, big, 8, 4096, 64, SM, big, big) == (False, big * 4096)
+
+
+@pytest.mark.parametrize("docs,branches,tokens,G,Hkv", [(1, 96, 128, 4, 8), (4, 96, 300, 4, 8), (1, 6144, 128, 4, 8), (18, 200, 200, 1, 8)])
+def test_calls_without_the_steps_tokens_have_nothing_to_copy(rule, docs, branches, tokens, G, Hkv):
+    """A block's pass over all rows below it (measured 5 to 18 % slower with copy warps)."""
+    assert rule(docs, docs * branches, docs * tokens, G, Hkv, 128, SM, CAP, CAP)[0]
+    assert not rule(docs, docs * branches, docs * tokens, G, Hkv, 128, SM, CAP, CAP, new_tokens=0)[0]

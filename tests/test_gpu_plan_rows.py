@@ -75,7 +75,7 @@ def test_tables_moved_after_the_list_was_made(name):
     gen = torch.Generator(device="cuda").manual_seed(docs)
     rnd = lambda *s: torch.randn(*s, device="cuda", generator=gen).to(torch.bfloat16)                 # noqa: E731
     q, pk, pv, sk, sv = rnd(n, Hq, D), rnd(T, Hkv, D), rnd(T, Hkv, D), rnd(n * cap, Hkv, D), rnd(n * cap, Hkv, D)
-    depth, alive = dev(rng.integers(0, cap + 1, n).astype(np.int32)), dev(np.ones(n, np.uint8))
+    depth, alive = dev(rng.integers(0, cap, n).astype(np.int32)), dev(np.ones(n, np.uint8))
     vis = dev(rng.integers(0, np.repeat(L, cnt) + 1).astype(np.int32))
     m = B.MetaTables.alloc(g, docs + 1, n, T)
     if order:
@@ -86,9 +86,9 @@ def test_tables_moved_after_the_list_was_made(name):
     def attn(m, q, rows):
         o, lse = torch.zeros(rows, Hq, D, dtype=torch.bfloat16, device="cuda"), torch.zeros(rows, Hq, device="cuda")
         if order:
-            B.hpd_attn_decode_posorder(g, docs + 1, rows, n, T, q, pk, pv, sk, sv, dev(L), depth, alive, m, False, o, lse)
+            B.hpd_attn_decode_posorder(g, docs + 1, rows, n, T, q, pk, pv, sk, sv, dev(L), depth, alive, m, True, o, lse)
         else:
-            B.hpd_attn_decode(g, docs + 1, rows, n, T, q, pk, pv, sk, sv, dev(L), m, False, o, lse)
+            B.hpd_attn_decode(g, docs + 1, rows, n, T, q, pk, pv, sk, sv, dev(L), m, True, o, lse)
         torch.cuda.synchronize()
         return o, lse
 

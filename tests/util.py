@@ -31,7 +31,7 @@ def err_stats(got, want):
 
 def copy_warps_rule(build_dir):
     """The host rule that picks a decode launch's kernel, compiled from its header: f(n_docs, max_rows, total_prefix, G, Hkv, D, n_sm, work_cap,
-    part_cap) -> (copy warps, expected units)."""
+    part_cap, new_tokens = 1) -> (copy warps, expected units)."""
     import ctypes
     import os
     import subprocess
@@ -45,8 +45,8 @@ def copy_warps_rule(build_dir):
     fn = ctypes.CDLL(lib).rule
     fn.restype = ctypes.c_longlong
 
-    def call(*sizes):
+    def call(*sizes, new_tokens=1):
         pay = ctypes.c_int()
-        units = fn((ctypes.c_int * 9)(*sizes), ctypes.byref(pay))
+        units = fn((ctypes.c_int * 10)(*sizes, new_tokens), ctypes.byref(pay))
         return bool(pay.value), units
     return call
