@@ -609,8 +609,10 @@ hpd_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 }
                 if (t == 0) {
                     next_stage();
-                    if (kBeforeQ && ui > 0 && nt > 0) fetch_q();
-                    if (!ok) break;
+                    if constexpr (kBeforeQ) {
+                        if (ui > 0 && nt > 0) fetch_q();
+                        if (!ok) break;
+                    }
                 }
                 if (t >= 1) {
                     const int vs = vc % C::NV;
